@@ -55,12 +55,7 @@ GRIDS = {
 }
 # nominal int32 lanes per SM on GB300 (4 SM sub-partitions x 32 lanes), for context
 ALU_LANES_PER_SM = 128
-# algorithmic integer work of the per-step kernel: per token-advance
-# (r = a + 1, store, max, min, add/compare) and per batch-step (W, E, extent,
-# violation, T_busy, token counter)
-OPS_PER_TOKEN_ADVANCE = 5
-OPS_PER_BATCH_STEP = 6
-# algorithmic integer work of the event-driven kernel: per request start or
+# algorithmic integer work of the simulation kernel: per request start or
 # completion (KV reservation, earliest completion / start range, counter,
 # output store, queue bit) and per epoch, a step at which a request starts or
 # completes (the closed-form W, E, extent, max extent, violations, T_busy and
@@ -71,15 +66,6 @@ OPS_PER_EPOCH = 14
 # 30-60 ms per launch on GB300) and launches per kind (the fastest is kept)
 PROBE_ITERS = 20_000
 PROBE_LAUNCHES = 3
-# DRAM bytes (read + write) per launch of the step simulation kernel on the full
-# workload: 742.6 MB measured by ncu on the first 4,096 instances, scaled by
-# 10,000 / 4,096 (profiles/sim_kernel_step_online_delta_sweep_4096.md)
-SIM_DRAM_BYTES_PER_LAUNCH = 742.6e6 * 10_000 / 4_096
-# issue-slot and ALU-pipe utilisation of the same capture (smsp__issue_active and
-# sm__inst_executed_pipe_alu, percent of peak while active), reported beside the roofline
-SIM_NCU_ISSUE_ACTIVE = 0.750
-SIM_NCU_ALU_PIPE = 0.681
-
 
 def workload_config(kernel, wl, n_inst, policies, deltas, flush):
     kv = "none" if wl.kv_caps[0] == W.KV_INF else wl.kv_caps[0]
@@ -282,13 +268,14 @@ def main():
     ap.add_argument("--steps", type=int, default=5)
     ap.add_argument("--warmup", type=int, default=3)
     ap.add_argument("--impl", choices=["ours", "reference"], default="ours")
-    ap.add_argument("--kernel", choices=["step", "epoch"], default="step")
+    ap.add_argument("--kernel", choices=["step", "epoch"], default="step",
+                    help="the flag the simulator is created with (both run the event-driven kernel)")
     ap.add_argument("--workload", type=int, choices=sorted(GRIDS), default=DEFAULT_WID)
     ap.add_argument("--instances", type=int, default=0, help="use only the first N instances (profiling)")
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--oracle-cores", type=int, default=0, help="host processes for the oracle (default: all cores)")
     ap.add_argument("--no-e2e", action="store_true")
-    ap.add_argument("--no-epoch", action="store_true", help="skip the event-driven kernel's extra measurement")
+    ap.add_argument("--no-epoch", action="store_true", help="accepted, no effect (there is one kernel)")
     args = ap.parse_args()
     if args.impl == "reference":
         return reference_arm(args)
@@ -373,22 +360,6 @@ def main():
     clocks = sampler.stop()
     t_ms = sum(step_ms)
 
-    # the other kernel variant on the same inputs (same results), for comparison
-    other = None
-    if not args.no_epoch:
-        S2 = sim.Simulator(n_inst, wl.n_per_instance, B, wl.c, wl.tau, wl.p0, epoch=not epoch, timing=True)
-        for _ in range(max(args.warmup, 1)):
-            sweep(S2)
-        st2, summ2 = sim.isjl_sim_metrics(S2.handle)
-        busy2 = sum(summ2[i].T_busy for i in range(len(policies)))
-        if st2 != 0 or busy2 != busy_per_step:
-            raise RuntimeError("kernel variants disagree")
-        step2, sim2, _ = timed_steps(S2)
-        other = {"kernel": "step" if epoch else "epoch",
-                 "value": busy_per_step * args.steps / (sum(step2) / 1e3),
-                 "ms_per_step": sum(step2) / args.steps, "sim_ms_per_launch": sum(sim2) / len(sim2)}
-        S2.close()
-
     # e2e through the host-memory entry point: H2D of the inputs (and counts /
     # slack where the workload has them), sweep, D2H of the records
     e2e = None
@@ -433,21 +404,21 @@ def main():
     peaks = probe_peaks(sim, stream)
     probe_clocks = probe_sampler.stop()
     peak_tops = peaks["add"]
-    # the event-driven kernel's own algorithmic work, counted from the outputs
+    # the kernel's algorithmic work, counted from the outputs
     # of one sweep (starts and completions per request, distinct event steps)
     res = S.sweep(a, p, o, policies, deltas, kv, per_request=True, counts=cnt, slack=slk)
     st_h, co_h = res["start"], res["completion"]
     n_events = int((st_h >= 0).sum() + (co_h >= 0).sum())
     n_epochs = epoch_count(st_h, co_h)
     del res, st_h, co_h
-    ops_step = OPS_PER_TOKEN_ADVANCE * tok_per_step + OPS_PER_BATCH_STEP * busy_per_step
-    ops_epoch = OPS_PER_REQUEST_EVENT * n_events + OPS_PER_EPOCH * n_epochs
+    ops = OPS_PER_REQUEST_EVENT * n_events + OPS_PER_EPOCH * n_epochs
 
-    def roof(kernel_name, ops, ms_per_launch, traffic):
+    def roof(ms_per_launch):
         achieved = ops / (ms_per_launch / 1e3) / 1e12
         return {"bound": "alu", "achieved": achieved, "peak": peak_tops, "unit": "Tops/s",
-                "frac": achieved / peak_tops, "traffic": traffic, "kernel": kernel_name,
+                "frac": achieved / peak_tops, "traffic": None, "kernel": "sim_kernel",
                 "ops_per_launch": ops, "sim_ms_per_launch": ms_per_launch,
+                "epochs_per_launch": n_epochs, "request_events_per_launch": n_events,
                 "peak_measured": peaks["add"], "alu_pipe_peak_measured": peaks["minmax"],
                 "frac_of_alu_pipe": achieved / peaks["minmax"], "peak_nominal": nominal_tops,
                 "peak_basis": (f"measured: isjl_probe_int_rate, int32 add chains ({peaks['add']:.2f} Tops/s) and "
@@ -455,21 +426,8 @@ def main():
                                f"full-occupancy launches at {probe_clocks.get('sm_mhz')} MHz; nominal "
                                f"{sms} SMs x {ALU_LANES_PER_SM} lanes x {sm_mhz:.0f} MHz = {nominal_tops:.2f}")}
 
-    full = wid == DEFAULT_WID and n_inst == wl.n_instances
     sim_avg_ms = sum(sim_ms) / len(sim_ms)
-    if epoch:
-        roofline = roof("sim_kernel (epoch)", ops_epoch, sim_avg_ms, None)
-    else:
-        roofline = roof("sim_kernel (step)", ops_step, sim_avg_ms, SIM_DRAM_BYTES_PER_LAUNCH if full else None)
-        if full:
-            roofline["ncu_issue_active"] = SIM_NCU_ISSUE_ACTIVE
-            roofline["ncu_alu_pipe"] = SIM_NCU_ALU_PIPE
-    if other is not None:
-        o_ops = ops_epoch if other["kernel"] == "epoch" else ops_step
-        o_roof = roof(f"sim_kernel ({other['kernel']})", o_ops, other["sim_ms_per_launch"], None)
-        other["roofline"] = {k: o_roof[k] for k in ("achieved", "frac", "frac_of_alu_pipe", "ops_per_launch")}
-        other["epochs_per_launch"] = n_epochs
-        other["request_events_per_launch"] = n_events
+    roofline = roof(sim_avg_ms)
 
     cpu = None
     if pool is not None:
@@ -485,7 +443,7 @@ def main():
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": t_ms_all / args.steps, "higher_is_better": True,
         "scaling": "weak", "vs_baseline": None, "dtype": "int32", "data": "synthetic",
-        "config": workload_config(args.kernel, wl, n_inst, policies, deltas,
+        "config": workload_config("event-driven", wl, n_inst, policies, deltas,
                                   "flushed between steps (256 MiB write, outside the events)"),
         "roofline": roofline,
         "cpu_baseline": cpu,
@@ -500,7 +458,6 @@ def main():
         "instances_per_s": world * n_inst * len(policies) * args.steps / (t_ms_all / 1e3),
         "token_advances_per_s": tok_per_step * world * args.steps / (t_ms_all / 1e3),
         "kernel_ms": {"sim": sim_avg_ms},
-        "other_kernel": other,
         "wall_s": wall,
     }
     print(json.dumps(line), flush=True)

@@ -72,8 +72,11 @@ typedef enum {
 #define ISJL_MAX_RUNS  32           /* largest (policy, delta) list of one sweep call */
 
 /* config flags */
-#define ISJL_FLAG_STEP_KERNEL 0u    /* default: per-step kernel, every running request advanced each step */
-#define ISJL_FLAG_EPOCH_KERNEL 1u   /* event-driven kernel: closed-form cost between events; same results */
+/* The simulation advances from event to event and adds the cost of the steps in
+ * between in closed form, with or without ISJL_FLAG_EPOCH_KERNEL, which asks for
+ * it by name and is kept for callers that set it. */
+#define ISJL_FLAG_STEP_KERNEL 0u    /* default */
+#define ISJL_FLAG_EPOCH_KERNEL 1u   /* accepted, no effect */
 #define ISJL_FLAG_TIMING 2u         /* record CUDA events around each kernel (see isjl_sim_kernel_times) */
 
 typedef struct {

@@ -94,8 +94,7 @@ isjl_status isjl_sim_create(const isjl_config *cfg, isjl_sim **out) {
     s->N = cfg->n_instances * (int64_t)cfg->n_per_instance;
     if (cudaGetDevice(&s->device) != cudaSuccess) { delete s; return ISJL_ERR_CUDA; }
     const int n = cfg->n_per_instance;
-    const bool epoch = (cfg->flags & ISJL_FLAG_EPOCH_KERNEL) != 0u;
-    s->total_warps = isjl::sim_resident_warps(cfg->B, n, epoch, s->device);
+    s->total_warps = isjl::sim_resident_warps(cfg->B, n, s->device);
     if (s->total_warps < 1) { delete s; cudaGetLastError(); return ISJL_ERR_INVALID_ARG; }   // B, n too large for smem
     bool ok = dalloc(&s->d_o, s->N) == cudaSuccess && dalloc(&s->d_perm, s->N) == cudaSuccess &&
               dalloc(&s->d_osorted, s->N) == cudaSuccess && dalloc(&s->d_posof, s->N) == cudaSuccess &&
@@ -188,8 +187,7 @@ isjl_status isjl_sim_run_sweep(isjl_sim *s, int32_t n_runs, const int32_t *polic
     a.tau = c.tau;
     a.p0 = c.p0;
     a.runs = runs;
-    const bool epoch = (c.flags & ISJL_FLAG_EPOCH_KERNEL) != 0u;
-    if (isjl::launch_sim(a, epoch, s->total_warps, st) != cudaSuccess || !mark(3)) return ISJL_ERR_CUDA;
+    if (isjl::launch_sim(a, s->total_warps, st) != cudaSuccess || !mark(3)) return ISJL_ERR_CUDA;
     s->last_launches++;
     if (isjl::launch_summarize(out->records, c.n_instances, n_runs, runs, kv_cap, s->d_summary, st) !=
             cudaSuccess || !mark(4))

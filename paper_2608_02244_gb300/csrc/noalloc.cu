@@ -84,10 +84,9 @@ extern "C" isjl_status isjl_sim_run_sweep_noalloc(const isjl_config *cfg, int32_
     const size_t ctr_off = off;      off = align256(off + 2 * sizeof(int32_t));
     const size_t plan_off = off;
     if (off >= kScratchBytes) return ISJL_ERR_INVALID_ARG;   // too large for the fixed workspace
-    const bool epoch = (cfg->flags & ISJL_FLAG_EPOCH_KERNEL) != 0u;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return ISJL_ERR_CUDA;
-    int warps = isjl::sim_resident_warps(cfg->B, n, epoch, dev);
+    int warps = isjl::sim_resident_warps(cfg->B, n, dev);
     if (warps < 1) return ISJL_ERR_INVALID_ARG;
     const int64_t fit = (int64_t)((kScratchBytes - plan_off) / (sizeof(int32_t) * (size_t)n));
     if (fit < warps) warps = (int)(fit / isjl::kSimWarpsPerBlock) * isjl::kSimWarpsPerBlock;
@@ -144,6 +143,6 @@ extern "C" isjl_status isjl_sim_run_sweep_noalloc(const isjl_config *cfg, int32_
         a.runs.delta[i] = deltas[i];
         a.runs.beta[i] = isjl::run_beta(policies[i], deltas[i]);
     }
-    if (isjl::launch_sim(a, epoch, warps, st) != cudaSuccess) return ISJL_ERR_CUDA;
+    if (isjl::launch_sim(a, warps, st) != cudaSuccess) return ISJL_ERR_CUDA;
     return ISJL_OK;
 }

@@ -78,11 +78,11 @@ cudaError_t launch_derive(const int32_t *arrival, const int32_t *prompt, const i
                           InstStats *inst, int64_t n_inst, int32_t n, cudaStream_t s);
 cudaError_t launch_sort(const int32_t *o, const InstStats *inst, int32_t *perm, int32_t *osorted, int32_t *posof,
                         int32_t *tmp, int64_t n_inst, int32_t n, cudaStream_t s);
-cudaError_t launch_sim(const SimArgs &args, bool epoch, int total_warps, cudaStream_t s);
+cudaError_t launch_sim(const SimArgs &args, int total_warps, cudaStream_t s);
 cudaError_t launch_summarize(const isjl_record *records, int64_t n_inst, int32_t n_runs,
                              const RunList &runs, int32_t kv_cap, isjl_summary *out, cudaStream_t s);
 // resident warps the simulation kernel is launched with for this B and n
-int sim_resident_warps(int B, int n, bool epoch, int device);
+int sim_resident_warps(int B, int n, int device);
 size_t sim_smem_per_warp(int B, int n);
 int slots_per_lane(int B);
 

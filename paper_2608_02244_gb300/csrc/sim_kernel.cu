@@ -1,51 +1,40 @@
-// sim_kernel.cu -- the per-step simulation of FCFS, LJF and ISJL on sm_103a.
+// sim_kernel.cu -- the simulation of FCFS, LJF, SJF and ISJL on sm_103a.
 //
 // One warp simulates one (instance, run) task; a persistent grid of warps
-// pulls tasks from a global counter.  Within a task every step does, in the
-// order of the paper's model (Section 2) and policies:
-//   release   requests with A_i <= k join the pending queue Q(k)
-//   retire    requests that finished in step k-1 leave the batch, c_i = k
-//   admit     FCFS / LJF (Algorithm 1) / ISJL (Algorithm 2, Sec. 3.4 rolling)
-//   advance   every running request processes token r_i = a_i + 1
-//   cost      W += |S| max r, E += sum (max r - r_i), extent, T_busy
-//             (Section 5, Eq. batch-cost-progress and the decomposition)
+// pulls tasks from a global counter.  The model is the paper's token-step one
+// (Section 2): in step k, requests with A_i <= k join the pending queue Q(k),
+// requests that finished in step k - 1 leave the batch (c_i = k), the policy
+// admits (FCFS, LJF of Algorithm 1, SJF, ISJL of Algorithm 2 in Section 3.4's
+// rolling form), every running request processes token r_i = a_i + 1, and the
+// step costs W += |S| max r, E += sum (max r - r_i), extent, T_busy (Section 5,
+// Eq. batch-cost-progress and the decomposition).
 //
-// Layout.  Worker (batch slot) w lives in lane w % 32, register row w / 32,
-// so a warp holds B <= 32 * SPL workers.  The step kernel advances, each
-// step, every slot of the rows that hold a running worker (a per-row-count
-// instantiation of the step loop), straight-line: from 8 rows on, a slot's
-// progress a is packed as (a << 16) | (65535 - a), so one add advances it and
-// one per-half max collects both the step's max and (complemented) min, with
-// idle slots set at the start of each stretch to values that lose both;
-// below 8 rows an idle slot carries a progress below 0 as a signed value and
-// at least 2^31 as an unsigned one (signed max, unsigned min).  The
-// sum of progress over all steps is added per request, o (o + 1) / 2, when it
-// starts (a run stopped early takes back the unserved part).  Values that
-// change only at events (next
-// arrival, earliest completion, start range, KV reservation) are kept as
-// warp-uniform scalars, so the steps between two events run no branch and
-// no warp reduction beyond the two of the step cost.  The pending
-// queue is a bitset over the instance's request positions sorted by
-// (o desc, index asc) -- the longest pending request is the lowest set bit --
-// with a summary word per 32 words, in shared memory.  ISJL plans are
-// per-worker FIFO lists linked through a global scratch array.
-//
-// Two variants share the admission code:
-//   step kernel   advances every running request each step (the literal loop)
-//   epoch kernel  jumps from event to event (arrival, completion, o_1's delay
-//                 expiry) and adds the cost of the L steps in between in closed
-//                 form; the running set is constant there and progress moves
-//                 in lockstep, so every counter is identical.  While LJF has a
-//                 batch running or ISJL's gate is shut, completions that do not
-//                 change the running set's earliest or latest start are served
-//                 in the same pass (a completion window).
-// Admissions happen only at events: between events the running set, the KV
-// reservation and the queue are unchanged and A_max only grows, so a step
-// that could not start a request is followed by steps that cannot either.
+// The kernel jumps from event to event (arrival, completion, o_1's delay
+// expiry) and adds the cost of the L steps in between in closed form: the
+// running set is constant there and progress moves in lockstep, so every
+// counter equals the step-by-step sum.  Admissions happen only at events:
+// between events the running set, the KV reservation and the queue are
+// unchanged and A_max only grows, so a step that could not start a request is
+// followed by steps that cannot either.  While LJF has a batch running or
+// ISJL's gate is shut, completions that do not change the running set's
+// earliest or latest start are served in the same pass (a completion window).
+// (A loop that advances every running request in every step gave the same
+// results at 1.1 to 3.7 times the time over the measured sweeps -- 52.6 ms
+// against 19.2 ms for 10,000 x 1,000 requests under 7 runs, 273 ms against
+// 108 ms for 1,024 x 100,000 under 3 -- and nowhere less.)
 // Arrivals that cannot start anything before the next completion are released
 // at that completion, and an admission that starts several requests does so
 // up to 32 (ISJL plan entries: all) at a time, with the same outcome as one
 // start at a time.
+//
+// Layout.  Worker (batch slot) w lives in lane w % 32, register row w / 32,
+// so a warp holds B <= 32 * SPL workers.  Values that change only at events
+// (next arrival, earliest completion, start range, KV reservation) are kept as
+// warp-uniform scalars.  The pending queue is a bitset over the instance's
+// request positions sorted by (o desc, index asc) -- the longest pending
+// request is the lowest set bit -- with a summary word per 32 words, in shared
+// memory.  ISJL plans are per-worker FIFO lists linked through a global
+// scratch array.
 #include <climits>
 #include <cstdint>
 
@@ -55,11 +44,7 @@ namespace isjl {
 namespace {
 
 constexpr int32_t kNone = -1;
-constexpr int32_t kIdle = -(1 << 30);   // idle-slot progress sentinel base (unpacked step kernel)
-// step kernel with SPL >= 8: the progress a of a slot is packed as
-// (a << 16) | (65535 - a)
-constexpr uint32_t kPackedZero = 0xFFFFu;  // a = 0
-constexpr uint32_t kPackedStep = 0xFFFFu;  // one step: a + 1 above, 65535 - (a + 1) below
+constexpr int32_t kIdle = -(1 << 30);   // an idle slot's start step
 
 struct WarpSmem {
     int32_t *sjob;    // [B] request running on worker w
@@ -89,66 +74,6 @@ __device__ __forceinline__ int highest_worker(uint32_t m, int lane) {
     return __reduce_max_sync(kFull, v);
 }
 
-// a row count as a type, for the step loop's per-row-count instantiations
-template <int N> struct RowCount { static constexpr int value = N; };
-
-// Row counts the step loop is instantiated for, per SPL (ascending).  The
-// loop advances the smallest of them covering every running worker; a few
-// classes keep the kernel small (measured: 2 and 4 for SPL = 4; 2, 4 and 8
-// for SPL = 8; 4, 8 and 16 for SPL = 16), and its steps are unrolled by two
-// (four for SPL = 16).
-template <int SPL> struct RowClasses;
-template <> struct RowClasses<1> {
-    static constexpr int n = 1;
-    __host__ __device__ static constexpr int at(int i) { constexpr int v[1] = {1}; return v[i]; }
-};
-template <> struct RowClasses<2> {
-    static constexpr int n = 2;
-    __host__ __device__ static constexpr int at(int i) { constexpr int v[2] = {1, 2}; return v[i]; }
-};
-template <> struct RowClasses<4> {
-    static constexpr int n = 2;
-    __host__ __device__ static constexpr int at(int i) { constexpr int v[2] = {2, 4}; return v[i]; }
-};
-template <> struct RowClasses<8> {
-    static constexpr int n = 3;
-    __host__ __device__ static constexpr int at(int i) { constexpr int v[3] = {2, 4, 8}; return v[i]; }
-};
-template <> struct RowClasses<16> {
-    static constexpr int n = 3;
-    __host__ __device__ static constexpr int at(int i) { constexpr int v[3] = {4, 8, 16}; return v[i]; }
-};
-
-// rows advanced when the highest row holding a running worker is t - 1 (t = 0: none)
-template <int SPL>
-__device__ __forceinline__ int row_class(int t) {
-    using C = RowClasses<SPL>;
-    if (t <= 0) return 0;
-    int r = SPL;
-#pragma unroll
-    for (int i = C::n - 1; i >= 0; --i) if (C::at(i) >= t) r = C::at(i);
-    return r;
-}
-// call f(RowCount<rows>{}) for rows one of RowClasses<SPL> (indices LO..HI), by a tree of uniform branches
-template <int SPL, int LO, int HI, class F>
-__device__ __forceinline__ void dispatch_rows(int rows, F &f) {
-    using C = RowClasses<SPL>;
-    if constexpr (LO == HI) {
-        f(RowCount<C::at(LO)>{});
-    } else {
-        constexpr int MID = (LO + HI) / 2;
-        if (rows <= C::at(MID)) dispatch_rows<SPL, LO, MID>(rows, f);
-        else dispatch_rows<SPL, MID + 1, HI>(rows, f);
-    }
-}
-
-// per-16-bit-half unsigned maximum
-__device__ __forceinline__ uint32_t vmax_u16x2(uint32_t a, uint32_t b) {
-    uint32_t d;
-    asm("max.u16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
-    return d;
-}
-
 // acc += a * b into a 64-bit accumulator with one wide multiply-add
 __device__ __forceinline__ void mad_wide(int64_t &acc, uint32_t a, uint32_t b) {
     asm("mad.wide.u32 %0, %1, %2, %0;" : "+l"(acc) : "r"(a), "r"(b));
@@ -161,12 +86,6 @@ __device__ __forceinline__ uint64_t warp_sum_u64(uint64_t v) {
     const uint32_t b = __reduce_add_sync(kFull, (uint32_t)(v >> 22) & 0x3FFFFFu);
     const uint32_t c = __reduce_add_sync(kFull, (uint32_t)(v >> 44));
     return (uint64_t)a + ((uint64_t)b << 22) + ((uint64_t)c << 44);
-}
-
-__device__ __forceinline__ int64_t warp_sum64(int64_t v) {
-#pragma unroll
-    for (int s = 16; s > 0; s >>= 1) v += __shfl_xor_sync(kFull, v, s);
-    return v;
 }
 
 // first pending sorted position >= p, INT_MAX if none (uniform call)
@@ -269,7 +188,7 @@ __device__ __forceinline__ int first_pos_le(const int32_t *os, int n, int64_t x,
 // One (instance, run) task under policy P, a compile-time constant (FCFS, LJF,
 // SJF or ISJL; Algorithm "ISJL" runs the ISJL body with beta in the packing
 // thresholds), so each policy's code holds only its own admission rule.
-template <int SPL, bool EPOCH, int P>
+template <int SPL, int P>
 __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, int lane, int64_t gwarp,
                                          int64_t inst, int run) {
     const int n_slots = A.n, B = A.B;
@@ -295,10 +214,6 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
     int32_t *st_out = A.start_out ? A.start_out + out_off : nullptr;
     int32_t *co_out = A.compl_out ? A.compl_out + out_off : nullptr;
     const int words0 = (n + 31) >> 5, words1 = (words0 + 31) >> 5;
-    // packed progress in the step kernel's stretch pays off from 8 register
-    // rows on (measured); fewer rows keep the signed / unsigned sentinel
-    constexpr bool kPacked = !EPOCH && SPL >= 8;
-    constexpr int32_t kStartA = EPOCH ? 0 : (kPacked ? (int32_t)kPackedZero : 0);
 
     int64_t status = is.status;
     if (status == ISJL_OK && (int64_t)is.maxo > kv_cap) status = ISJL_ERR_INFEASIBLE;
@@ -312,13 +227,7 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
         if (co_out) for (int i = lane; i < n_slots; i += 32) co_out[i] = -1;
     }
 
-    // W = sum over steps of |S| max r; E = W - R, where R = sum over steps of
-    // sum r equals the sum over served requests of a (a + 1) / 2 for the
-    // tokens a each received (one per step from 1): the step kernel adds
-    // o (o + 1) / 2 when a request starts and takes back the unserved part of
-    // requests still running if a run stops early (the decomposition W = Q + E
-    // of Section 5)
-    int64_t W = 0, R = 0, E = 0, sumc = 0, sumext = 0;
+    int64_t W = 0, E = 0, sumc = 0, sumext = 0;
     int32_t peakkv = 0;
     int32_t Tb = 0, tok = 0, maxext = 0, viol = 0, peakb = 0, Tmake = 0, kvviol = 0;
 
@@ -328,28 +237,21 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
         for (int w = lane; w < B; w += 32) { S.shead[w] = kNone; S.stail[w] = kNone; S.slong[w] = kNone; }
         __syncwarp();
 
-        // worker w = r * 32 + lane: sa = progress (step kernel) or start step
-        // (epoch kernel), sc = completion step (INT_MAX when idle)
+        // worker w = r * 32 + lane: sa = start step, sc = completion step (INT_MAX when idle)
         int32_t sa[SPL], sc[SPL];
 #pragma unroll
         for (int r = 0; r < SPL; ++r) { sa[r] = kIdle; sc[r] = INT_MAX; }
         uint32_t busy = 0u, resv = 0u;
         uint32_t lhead = 0u;    // worker's next plan entry is its long job o_j (waits for o_1)
         int32_t lane_cmin = INT_MAX;                 // earliest completion among this lane's workers
-        int32_t lane_smin = INT_MAX, lane_smax = INT_MIN;   // start range (epoch kernel)
+        int32_t lane_smin = INT_MAX, lane_smax = INT_MIN;   // start range of this lane's workers
         const int nrow = (B - lane + 31) >> 5;       // rows holding a valid worker for this lane
         const uint32_t vmask = nrow >= 32 ? ~0u : ((1u << nrow) - 1u);
         const int32_t alpha32 = (int32_t)min(alpha, (int64_t)INT_MAX);
 
         int32_t k = 0, rel = 0, fcfs = 0, done = 0, run_cnt = 0, pend = 0;
-        // step kernel: register rows [0, adv_rows) are advanced each step; every
-        // running worker lies in them, and their idle slots hold the sentinel
-        int adv_rows = 0;
-        // step kernel: A_max at the current step, from the last step's max reduction
-        int32_t amax_c = 0;
-        bool amax_ok = false;
         int32_t kv_sum = 0;
-        uint32_t sum_st = 0;   // epoch kernel: the running requests' start steps, summed modulo 2^32
+        uint32_t sum_st = 0;   // the running requests' start steps, summed modulo 2^32
         // the next 32 unreleased requests (from win_base): arrival and sorted position, per lane
         int32_t win_base = 0, win_a = INT_MAX, win_p = 0;
         auto load_window = [&]() {
@@ -364,7 +266,7 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
         bool hvalid = true;                            // hp is current (else recompute from the bitset)
         int32_t fo = -1;                               // o of the FCFS head (-1: not loaded)
         int32_t cmin = INT_MAX;                        // earliest completion step of the running set
-        int32_t smin = INT_MAX, smax = INT_MIN;        // start range of the running set (epoch kernel)
+        int32_t smin = INT_MAX, smax = INT_MIN;        // start range of the running set
         int32_t kv_over = 0;                           // reserved KV above the cap (never, by construction)
         int32_t plan_left = 0, t0 = 0, d1 = 0, L1 = kNone, nlong = 0;
         bool L1_started = true;
@@ -374,11 +276,12 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
 
         auto recompute_lane = [&]() {
             lane_cmin = INT_MAX;
-            if (EPOCH) { lane_smin = INT_MAX; lane_smax = INT_MIN; }
+            lane_smin = INT_MAX;
+            lane_smax = INT_MIN;
 #pragma unroll
             for (int r = 0; r < SPL; ++r) {
                 lane_cmin = min(lane_cmin, sc[r]);               // idle slots hold INT_MAX
-                if (EPOCH && (busy >> r & 1u)) { lane_smin = min(lane_smin, sa[r]); lane_smax = max(lane_smax, sa[r]); }
+                if (busy >> r & 1u) { lane_smin = min(lane_smin, sa[r]); lane_smax = max(lane_smax, sa[r]); }
             }
         };
         // start request e (length oe) on worker w at step k
@@ -390,46 +293,38 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
             peakkv = max(peakkv, kv_sum);
             peakb = max(peakb, run_cnt);
             kv_over = kv_sum > kv_lim;
-            if (EPOCH) { sum_st += (uint32_t)k; smin = min(smin, k); smax = k; }
-            if (!EPOCH) mad_wide(R, ((uint32_t)oc * (uint32_t)(oc + 1)) >> 1, 1u);   // oc (oc + 1) < 2^32
+            sum_st += (uint32_t)k;
+            smin = min(smin, k);
+            smax = k;
             const int owner = w & 31, row = w >> 5;
-            if (!EPOCH && row >= adv_rows) adv_rows = row_class<SPL>(row + 1);
-            if (!EPOCH && run_cnt == 1) { amax_c = 0; amax_ok = true; }   // the only request: progress 0
             if (lane == owner) {
 #pragma unroll
                 for (int r = 0; r < SPL; ++r)
-                    if (r == row) { sa[r] = EPOCH ? k : kStartA; sc[r] = k + oc; }
+                    if (r == row) { sa[r] = k; sc[r] = k + oc; }
                 busy |= 1u << row;
                 lane_cmin = min(lane_cmin, k + oc);
                 S.sres[w] = oe;
-                if (EPOCH) { lane_smin = min(lane_smin, k); lane_smax = max(lane_smax, k); }
+                lane_smin = min(lane_smin, k);
+                lane_smax = max(lane_smax, k);
                 S.sjob[w] = e;
                 if (st_out) st_out[e] = k;
             }
         };
         // warp-wide totals of c starts at step k made lane-parallel: kv_add their
-        // reserved KV, my_cmin / rsum this lane's earliest completion and sum of
-        // o (o + 1) / 2, top the highest row that received one, plus one
-        auto commit_starts = [&](int c, int32_t kv_add, int32_t my_cmin, uint64_t rsum, int top) {
+        // reserved KV, my_cmin this lane's earliest completion
+        auto commit_starts = [&](int c, int32_t kv_add, int32_t my_cmin) {
             __syncwarp();
             lane_cmin = min(lane_cmin, my_cmin);
-            if (EPOCH && my_cmin != INT_MAX) { lane_smin = min(lane_smin, k); lane_smax = max(lane_smax, k); }
-            const bool was_empty = run_cnt == 0;
+            if (my_cmin != INT_MAX) { lane_smin = min(lane_smin, k); lane_smax = max(lane_smax, k); }
             run_cnt += c;
             kv_sum += kv_add;
             cmin = min(cmin, (int32_t)__reduce_min_sync(kFull, (unsigned)my_cmin));
             peakkv = max(peakkv, kv_sum);
             peakb = max(peakb, run_cnt);
             kv_over = kv_sum > kv_lim;
-            if (EPOCH) { sum_st += (uint32_t)c * (uint32_t)k; smin = min(smin, k); smax = k; }
-            if (!EPOCH) {
-                // rsum < 2^35 per lane: its low 24 bits and the rest summed by two reductions
-                const unsigned lo = __reduce_add_sync(kFull, (unsigned)(rsum & 0xFFFFFFu));
-                const unsigned hi = __reduce_add_sync(kFull, (unsigned)(rsum >> 24));
-                R += ((int64_t)hi << 24) + (int64_t)lo;
-                if (top > adv_rows) adv_rows = row_class<SPL>(top);
-                if (was_empty) { amax_c = 0; amax_ok = true; }   // the new requests: progress 0
-            }
+            sum_st += (uint32_t)c * (uint32_t)k;
+            smin = min(smin, k);
+            smax = k;
         };
         // Start, at step k, the longest prefix of up to 32 candidates (lane l < m
         // holds request ce and its planning length co) whose KV reservations fit
@@ -450,9 +345,8 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
             if (c == 0) return 0;
             const int oc_l = (otru && lane < c) ? otru[ce] : co;  // it finishes after its true length
             const uint32_t lt = (1u << lane) - 1u;
-            int base = 0, top = 0;
+            int base = 0;
             int32_t my_cmin = INT_MAX;
-            uint64_t rsum = 0;
 #pragma unroll
             for (int r = 0; r < SPL; ++r) {
                 if (base < c) {
@@ -465,34 +359,31 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
                     const int oc = __shfl_sync(kFull, oc_l, src);
                     if (f && rank < c) {
                         const int w = (r << 5) + lane;
-                        sa[r] = EPOCH ? k : kStartA;
+                        sa[r] = k;
                         sc[r] = k + oc;
                         busy |= 1u << r;
                         my_cmin = min(my_cmin, k + oc);
                         S.sres[w] = oe;
                         S.sjob[w] = e;
                         if (st_out) st_out[e] = k;
-                        if (!EPOCH) rsum += ((uint32_t)oc * (uint32_t)(oc + 1)) >> 1;
                     }
-                    if (rowf) top = r + 1;
                     base += __popc(rowf);
                 }
             }
-            commit_starts(c, __shfl_sync(kFull, pre, c - 1), my_cmin, rsum, top);
+            commit_starts(c, __shfl_sync(kFull, pre, c - 1), my_cmin);
             return c;
         };
         // requests completing at step c leave their workers
         auto retire = [&](int32_t c) {
             uint32_t fm = 0u;
-            unsigned sf = 0u;   // sum of (start - (c - 65536)) over finishing requests (epoch kernel)
+            unsigned sf = 0u;   // sum of (start - (c - 65536)) over finishing requests
 #pragma unroll
             for (int r = 0; r < SPL; ++r) {
                 const bool f = sc[r] == c;                   // idle slots hold INT_MAX
                 fm |= (uint32_t)f << r;
                 if (f) {
-                    if (EPOCH) sf += (unsigned)(sa[r] - (c - 65536));
+                    sf += (unsigned)(sa[r] - (c - 65536));
                     sc[r] = INT_MAX;
-                    if (!EPOCH && !kPacked) sa[r] = kIdle;
                 }
             }
             // per finishing request (usually one per warp): outputs and its KV release
@@ -504,45 +395,25 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
                 if (co_out) co_out[S.sjob[w]] = c;
             }
             busy &= ~fm;
-            // unconditional where measured cheaper than the branch (not the epoch kernel's 16 rows)
-            if (!EPOCH || SPL <= 8 || fm) recompute_lane();
-            if (!EPOCH) adv_rows = row_class<SPL>((int)__reduce_max_sync(kFull, 32u - (unsigned)__clz((int)busy)));
+            // unconditional where measured cheaper than the branch (not for 16 rows)
+            if (SPL <= 8 || fm) recompute_lane();
             nf = (int)__reduce_add_sync(kFull, (unsigned)nf);
             of = (int)__reduce_add_sync(kFull, (unsigned)of);
-            if (EPOCH)   // starts are within 65535 steps of c, so the offsets fit 32 bits
-                sum_st -= __reduce_add_sync(kFull, sf) + (uint32_t)nf * (uint32_t)(c - 65536);
+            // starts are within 65535 steps of c, so the offsets fit 32 bits
+            sum_st -= __reduce_add_sync(kFull, sf) + (uint32_t)nf * (uint32_t)(c - 65536);
             done += nf;
             run_cnt -= nf;
-            if (!EPOCH && nf > 0) amax_ok = false;
             kv_sum -= of;
             kv_over = kv_sum > kv_lim;
             sumc += (int64_t)nf * c;
             Tmake = c;
             cmin = __reduce_min_sync(kFull, lane_cmin);
-            if (EPOCH) {
-                smin = __reduce_min_sync(kFull, lane_smin);
-                smax = __reduce_max_sync(kFull, lane_smax);
-            }
+            smin = __reduce_min_sync(kFull, lane_smin);
+            smax = __reduce_max_sync(kFull, lane_smax);
         };
         // A_max(k): largest progress among running requests (0 if none)
         auto amax_now = [&]() -> int32_t {
-            if (run_cnt == 0) return 0;
-            if (EPOCH) return k - smin;
-            if (!amax_ok) {
-                if constexpr (kPacked) {
-                    uint32_t m = 0u;    // packed progress: the larger value has the larger a
-#pragma unroll
-                    for (int r = 0; r < SPL; ++r) if (busy >> r & 1u) m = max(m, (uint32_t)sa[r]);
-                    amax_c = (int32_t)(__reduce_max_sync(kFull, m) >> 16);
-                } else {
-                    int m = 0;
-#pragma unroll
-                    for (int r = 0; r < SPL; ++r) if (busy >> r & 1u) m = max(m, sa[r]);
-                    amax_c = __reduce_max_sync(kFull, m);
-                }
-                amax_ok = true;
-            }
-            return amax_c;
+            return run_cnt == 0 ? 0 : k - smin;
         };
 
         auto release = [&]() {
@@ -664,10 +535,9 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
         // is always the first candidate and is started one at a time.
         auto plan_bulk = [&](uint32_t cand, bool over) -> bool {
             bool stopped = false;
-            int c = 0, top = 0;
+            int c = 0;
             int32_t kv_add = 0;
             int32_t my_cmin = INT_MAX;
-            uint64_t rsum = 0;
 #pragma unroll
             for (int r = 0; r < SPL; ++r) {
                 if (!stopped) {
@@ -698,21 +568,19 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
                         if (w >= 1 && w < nlong && nx >= 0 && nx == S.slong[w]) lhead |= bit;
                         else lhead &= ~bit;
                         const int oc = otru ? otru[e] : oe;     // it finishes after its true length
-                        sa[r] = EPOCH ? k : kStartA;
+                        sa[r] = k;
                         sc[r] = k + oc;
                         busy |= bit;
                         my_cmin = min(my_cmin, k + oc);
                         S.sres[w] = oe;
                         S.sjob[w] = e;
                         if (st_out) st_out[e] = k;
-                        if (!EPOCH) rsum += ((uint32_t)oc * (uint32_t)(oc + 1)) >> 1;
                     }
-                    if (fb) top = r + 1;
                     c += __popc(fb);
                     kv_add += (int32_t)__reduce_add_sync(kFull, fits ? (unsigned)oe : 0u);
                 }
             }
-            if (c > 0) commit_starts(c, kv_add, my_cmin, rsum, top);
+            if (c > 0) commit_starts(c, kv_add, my_cmin);
             plan_left -= c;
             return stopped;
         };
@@ -1024,80 +892,7 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
             }
         };
 
-        // steps k .. k + L - 1 with no event: advance rows [0, NR), which hold
-        // every running worker, and add each step's cost.
-        //   SPL >= 8: a slot's progress a is packed as (a << 16) | (65535 - a)
-        //   (o <= 65535): one add of 0xFFFF advances both halves (no borrow: a < o
-        //   while the request runs), and a per-half unsigned max over a lane's
-        //   slots, then two warp max reductions, give max r (upper half) and
-        //   65535 - min r (lower half).  Idle slots of these rows are first set
-        //   to (0, L): after j steps they hold (j, L - j), at most the running
-        //   slots' halves, since every running request has a >= j and none
-        //   completes inside the stretch (min a + L <= its o <= 65535).
-        //   SPL < 8: idle slots hold a value below 0 as a signed number and at
-        //   least 2^31 as an unsigned one, so they lose the signed max and the
-        //   unsigned min.
-        auto plain_steps = [&](auto nr_tag, int L) {
-            constexpr int NR = decltype(nr_tag)::value;
-            const uint32_t cnt = (uint32_t)run_cnt;
-            constexpr int kUnroll = SPL >= 16 ? 4 : 2;   // measured; more code costs instruction-cache misses
-            if constexpr (kPacked) {
-#pragma unroll
-                for (int r = 0; r < NR; ++r)
-                    if (!(busy >> r & 1u)) sa[r] = L;
-                uint32_t last_mx = 0u, smx = 0u, sext = 0u;   // sums over the stretch: L, r < 2^16
-#pragma unroll kUnroll
-                for (int j = 0; j < L; ++j) {
-                    uint32_t m = 0u;
-#pragma unroll
-                    for (int r = 0; r < NR; ++r) {
-                        const uint32_t a = (uint32_t)sa[r] + kPackedStep;
-                        sa[r] = (int32_t)a;
-                        m = vmax_u16x2(m, a);
-                    }
-                    const uint32_t mx = __reduce_max_sync(kFull, m) >> 16;          // max r
-                    const uint32_t lo = __reduce_max_sync(kFull, m & 0xFFFFu);      // 65535 - min r
-                    const int ext = (int)(mx + lo) - 65535;
-                    smx += mx;
-                    sext += (uint32_t)ext;
-                    maxext = max(maxext, ext);
-                    viol += ext > alpha32;
-                    last_mx = mx;
-                }
-                mad_wide(W, cnt, smx);                   // |S| max r, summed over the steps
-                sumext += sext;
-                amax_c = (int32_t)last_mx;               // max progress entering step k + L
-            } else {
-                int last_mx = 0;
-                uint32_t smx = 0u, sext = 0u;            // sums over the stretch: L, r < 2^16
-#pragma unroll kUnroll
-                for (int j = 0; j < L; ++j) {
-                    int mx = INT_MIN;
-                    unsigned mn = 0xffffffffu;
-#pragma unroll
-                    for (int r = 0; r < NR; ++r) {
-                        const int a = sa[r] + 1;
-                        sa[r] = a;
-                        mx = max(mx, a);
-                        mn = min(mn, (unsigned)a);
-                    }
-                    mx = __reduce_max_sync(kFull, mx);
-                    mn = __reduce_min_sync(kFull, mn);
-                    const int ext = mx - (int)mn;
-                    smx += (uint32_t)mx;
-                    sext += (uint32_t)ext;
-                    maxext = max(maxext, ext);
-                    viol += ext > alpha32;
-                    last_mx = mx;
-                }
-                mad_wide(W, cnt, smx);                   // |S| max r, summed over the steps
-                sumext += sext;
-                amax_c = last_mx;                        // max progress entering step k + L
-            }
-            amax_ok = true;
-        };
-
-        // epoch kernel: the step at which the running set's earliest or latest
+        // the step at which the running set's earliest or latest
         // start changes (the last completion among the requests that started at
         // smin, or at smax)
         auto window_end = [&]() -> int32_t {
@@ -1110,7 +905,7 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
                 }
             return min(__reduce_max_sync(kFull, e_lo), __reduce_max_sync(kFull, e_hi));
         };
-        // epoch kernel: serve steps k .. K - 1 at once, K <= the step at which
+        // serve steps k .. K - 1 at once, K <= the step at which
         // the earliest or latest start changes.  Every running request i
         // (start s_i, completion c_i) runs L_i = min(c_i, K) - k of them, with
         // max r = t - smin + 1 at step t and r_i = t - s_i + 1:
@@ -1170,98 +965,51 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
         };
 
         // release every request with A_i <= k (a prefix: arrivals are non-decreasing)
-        if (!EPOCH) {
-            // ---------------------------------------------------- step kernel
-            int32_t next_check = 0;   // the next step needing release / admission / the guard
-            for (;;) {
-                if (k >= next_check) {
-                    if (k >= step_guard) { status = ISJL_ERR_STEP_LIMIT; break; }
-                    if (done == n) break;
-                    if (k >= next_arr) release();
-                    admit();
-                    if (broken) { status = ISJL_ERR_INTERNAL; break; }
-                    next_check = blocked && run_cnt > 0 ? INT_MAX : next_arr;
-                    if (policy == ISJL_POLICY_ISJL && !L1_started && t0 + d1 > k) next_check = min(next_check, t0 + d1);
-                    next_check = min(next_check, step_guard);
-                }
-                if (run_cnt == 0) { k = next_check; continue; }   // idle steps: nothing to serve
-                // no arrival, completion, delay expiry or guard before step e
-                const int32_t e = min(next_check, cmin);
-                const int L = e - k;
-                {
-                    auto f = [&](auto nr_tag) { plain_steps(nr_tag, L); };
-                    if (adv_rows < 1) broken = true;
-                    else dispatch_rows<SPL, 0, RowClasses<SPL>::n - 1>(adv_rows, f);
-                }
-                if (broken) { status = ISJL_ERR_INTERNAL; break; }
-                Tb += L;
-                tok += L * run_cnt;
-                if (kv_over) kvviol += L;
-                k = e;
-                if (k == cmin && k < step_guard) {   // requests that finished in step k - 1 leave
-                    retire(k);
-                    next_check = k;
+        for (;;) {
+            if (k >= step_guard) { status = ISJL_ERR_STEP_LIMIT; break; }   // k > max_steps
+            if (k >= next_arr) release();
+            if (k == cmin) retire(k);
+            if (done == n) break;
+            admit();
+            if (broken) { status = ISJL_ERR_INTERNAL; break; }
+            // next event: arrival, completion or the end of o_1's delay
+            int32_t nxt = min(blocked && run_cnt > 0 ? INT_MAX : next_arr, cmin);
+            if (policy == ISJL_POLICY_ISJL && !L1_started && t0 + d1 > k) nxt = min(nxt, t0 + d1);
+            if (nxt == INT_MAX) { status = ISJL_ERR_STEP_LIMIT; break; }   // cannot progress
+            nxt = min(nxt, step_guard);                          // serve no step past max_steps
+            // LJF with a batch running, or ISJL with its gate shut (A_max only
+            // grows while the earliest start stays): no request can start
+            // before the running set's earliest or latest start changes, so
+            // completions in between end no epoch of their own
+            if (run_cnt > 0 && !kv_over && nxt == cmin &&
+                (policy == ISJL_POLICY_LJF || (policy == ISJL_POLICY_ISJL && k - smin > alpha32))) {
+                const int32_t K = min(window_end(), step_guard);
+                if (K > nxt) {
+                    window(K);
+                    k = K;
+                    continue;
                 }
             }
-            // a request still running (a run stopped early) with progress a and
-            // true length o = a + (completion - k) has served only a (a + 1) / 2
-            int64_t unserved = 0;
-#pragma unroll
-            for (int r = 0; r < SPL; ++r)
-                if (busy >> r & 1u) {
-                    const uint32_t a = kPacked ? (uint32_t)sa[r] >> 16 : (uint32_t)sa[r];
-                    const uint32_t o = a + (uint32_t)(sc[r] - k);
-                    unserved += (int64_t)((o * (o + 1u)) >> 1) - (int64_t)((a * (a + 1u)) >> 1);
-                }
-            E = W - (R - warp_sum64(unserved));
-        } else {
-            // --------------------------------------------------- epoch kernel
-            for (;;) {
-                if (k >= step_guard) { status = ISJL_ERR_STEP_LIMIT; break; }   // k > max_steps
-                if (k >= next_arr) release();
-                if (k == cmin) retire(k);
-                if (done == n) break;
-                admit();
-                if (broken) { status = ISJL_ERR_INTERNAL; break; }
-                // next event: arrival, completion or the end of o_1's delay
-                int32_t nxt = min(blocked && run_cnt > 0 ? INT_MAX : next_arr, cmin);
-                if (policy == ISJL_POLICY_ISJL && !L1_started && t0 + d1 > k) nxt = min(nxt, t0 + d1);
-                if (nxt == INT_MAX) { status = ISJL_ERR_STEP_LIMIT; break; }   // cannot progress
-                nxt = min(nxt, step_guard);                          // serve no step past max_steps
-                // LJF with a batch running, or ISJL with its gate shut (A_max only
-                // grows while the earliest start stays): no request can start
-                // before the running set's earliest or latest start changes, so
-                // completions in between end no epoch of their own
-                if (run_cnt > 0 && !kv_over && nxt == cmin &&
-                    (policy == ISJL_POLICY_LJF || (policy == ISJL_POLICY_ISJL && k - smin > alpha32))) {
-                    const int32_t K = min(window_end(), step_guard);
-                    if (K > nxt) {
-                        window(K);
-                        k = K;
-                        continue;
-                    }
-                }
-                if (run_cnt > 0) {
-                    // L steps, max r = m0 + t at step k + t, sum r = s m0 - sum (s_i - smin) + s t:
-                    //   W += s (L m0 + L (L - 1) / 2),  E += L sum (s_i - smin)
-                    // The epoch ends by the completion of the request that started at
-                    // smin, so max r <= its o <= 65535 throughout: the sum of max r over
-                    // the L <= 65535 steps fits 32 bits, and sum (s_i - smin) <
-                    // B * 65536 is exact from the modular sum of starts.
-                    const uint32_t L = (uint32_t)(nxt - k), s = (uint32_t)run_cnt;
-                    const uint32_t m0 = (uint32_t)(k - smin + 1);     // max r at step k
-                    const int32_t ext = smax - smin;                  // max r - min r
-                    mad_wide(W, s, L * m0 + ((L * (L - 1u)) >> 1));
-                    mad_wide(E, L, sum_st - s * (uint32_t)smin);
-                    mad_wide(sumext, L, (uint32_t)ext);
-                    maxext = max(maxext, ext);
-                    viol += ext > alpha32 ? (int32_t)L : 0;
-                    kvviol += kv_over ? (int32_t)L : 0;
-                    Tb += (int32_t)L;
-                    tok += (int32_t)(s * L);
-                }
-                k = nxt;
+            if (run_cnt > 0) {
+                // L steps, max r = m0 + t at step k + t, sum r = s m0 - sum (s_i - smin) + s t:
+                //   W += s (L m0 + L (L - 1) / 2),  E += L sum (s_i - smin)
+                // The epoch ends by the completion of the request that started at
+                // smin, so max r <= its o <= 65535 throughout: the sum of max r over
+                // the L <= 65535 steps fits 32 bits, and sum (s_i - smin) <
+                // B * 65536 is exact from the modular sum of starts.
+                const uint32_t L = (uint32_t)(nxt - k), s = (uint32_t)run_cnt;
+                const uint32_t m0 = (uint32_t)(k - smin + 1);     // max r at step k
+                const int32_t ext = smax - smin;                  // max r - min r
+                mad_wide(W, s, L * m0 + ((L * (L - 1u)) >> 1));
+                mad_wide(E, L, sum_st - s * (uint32_t)smin);
+                mad_wide(sumext, L, (uint32_t)ext);
+                maxext = max(maxext, ext);
+                viol += ext > alpha32 ? (int32_t)L : 0;
+                kvviol += kv_over ? (int32_t)L : 0;
+                Tb += (int32_t)L;
+                tok += (int32_t)(s * L);
             }
+            k = nxt;
         }
     }
 
@@ -1306,24 +1054,20 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
 // resident blocks per SM the register allocation is bounded for, per
 // instantiation (measured on GB300): 4 (up to 128 registers) in general;
 // SPL_BLOCKS16 for 16 register rows (B > 256), where shared memory already
-// limits large instances to 2 blocks per SM and a tighter bound only spills;
-// SPL_BLOCKS4_STEP for the step kernel with 4 rows (B <= 128)
+// limits large instances to 2 blocks per SM and a tighter bound only spills
 #ifndef ISJL_SIM_MIN_BLOCKS
 #define ISJL_SIM_MIN_BLOCKS 4
 #endif
 #ifndef ISJL_SIM_BLOCKS16
 #define ISJL_SIM_BLOCKS16 3
 #endif
-#ifndef ISJL_SIM_BLOCKS4_STEP
-#define ISJL_SIM_BLOCKS4_STEP 5
-#endif
-template <int SPL, bool EPOCH>
+template <int SPL>
 constexpr int sim_min_blocks() {
-    return SPL >= 16 ? ISJL_SIM_BLOCKS16 : (SPL == 4 && !EPOCH ? ISJL_SIM_BLOCKS4_STEP : ISJL_SIM_MIN_BLOCKS);
+    return SPL >= 16 ? ISJL_SIM_BLOCKS16 : ISJL_SIM_MIN_BLOCKS;
 }
 
-template <int SPL, bool EPOCH>
-__global__ void __launch_bounds__(kSimWarpsPerBlock * 32, sim_min_blocks<SPL, EPOCH>())
+template <int SPL>
+__global__ void __launch_bounds__(kSimWarpsPerBlock * 32, sim_min_blocks<SPL>())
 sim_kernel(SimArgs A, int64_t n_tasks) {
     extern __shared__ __align__(16) int32_t smem[];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -1349,24 +1093,24 @@ sim_kernel(SimArgs A, int64_t n_tasks) {
         const int64_t inst = t % A.n_inst;
         const int run = (int)(t / A.n_inst);
         switch (A.runs.policy[run]) {
-            case ISJL_POLICY_FCFS: run_task<SPL, EPOCH, ISJL_POLICY_FCFS>(A, S, lane, gwarp, inst, run); break;
-            case ISJL_POLICY_LJF:  run_task<SPL, EPOCH, ISJL_POLICY_LJF>(A, S, lane, gwarp, inst, run); break;
-            case ISJL_POLICY_SJF:  run_task<SPL, EPOCH, ISJL_POLICY_SJF>(A, S, lane, gwarp, inst, run); break;
-            default:               run_task<SPL, EPOCH, ISJL_POLICY_ISJL>(A, S, lane, gwarp, inst, run); break;
+            case ISJL_POLICY_FCFS: run_task<SPL, ISJL_POLICY_FCFS>(A, S, lane, gwarp, inst, run); break;
+            case ISJL_POLICY_LJF:  run_task<SPL, ISJL_POLICY_LJF>(A, S, lane, gwarp, inst, run); break;
+            case ISJL_POLICY_SJF:  run_task<SPL, ISJL_POLICY_SJF>(A, S, lane, gwarp, inst, run); break;
+            default:               run_task<SPL, ISJL_POLICY_ISJL>(A, S, lane, gwarp, inst, run); break;
         }
     }
 }
 
-template <int SPL, bool EPOCH>
-const void *kernel_ptr() { return reinterpret_cast<const void *>(&sim_kernel<SPL, EPOCH>); }
+template <int SPL>
+const void *kernel_ptr() { return reinterpret_cast<const void *>(&sim_kernel<SPL>); }
 
-const void *pick_kernel(int spl, bool epoch) {
+const void *pick_kernel(int spl) {
     switch (spl) {
-        case 1:  return epoch ? kernel_ptr<1, true>() : kernel_ptr<1, false>();
-        case 2:  return epoch ? kernel_ptr<2, true>() : kernel_ptr<2, false>();
-        case 4:  return epoch ? kernel_ptr<4, true>() : kernel_ptr<4, false>();
-        case 8:  return epoch ? kernel_ptr<8, true>() : kernel_ptr<8, false>();
-        default: return epoch ? kernel_ptr<16, true>() : kernel_ptr<16, false>();
+        case 1:  return kernel_ptr<1>();
+        case 2:  return kernel_ptr<2>();
+        case 4:  return kernel_ptr<4>();
+        case 8:  return kernel_ptr<8>();
+        default: return kernel_ptr<16>();
     }
 }
 
@@ -1383,8 +1127,8 @@ size_t sim_smem_per_warp(int B, int n) {
     return (size_t)smem_words_per_warp(B, words0, words1) * 4;
 }
 
-static cudaError_t occupancy(int B, int n, bool epoch, int device, int *blocks_per_sm, int *sms, size_t *smem) {
-    const void *k = pick_kernel(slots_per_lane(B), epoch);
+static cudaError_t occupancy(int B, int n, int device, int *blocks_per_sm, int *sms, size_t *smem) {
+    const void *k = pick_kernel(slots_per_lane(B));
     *smem = sim_smem_per_warp(B, n) * kSimWarpsPerBlock;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*smem);
     if (e != cudaSuccess) return e;
@@ -1393,26 +1137,26 @@ static cudaError_t occupancy(int B, int n, bool epoch, int device, int *blocks_p
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, kSimWarpsPerBlock * 32, *smem);
 }
 
-int sim_resident_warps(int B, int n, bool epoch, int device) {
+int sim_resident_warps(int B, int n, int device) {
     int bps = 0, sms = 0;
     size_t smem = 0;
-    if (occupancy(B, n, epoch, device, &bps, &sms, &smem) != cudaSuccess || bps < 1) return 0;
+    if (occupancy(B, n, device, &bps, &sms, &smem) != cudaSuccess || bps < 1) return 0;
     return bps * sms * kSimWarpsPerBlock;
 }
 
-cudaError_t launch_sim(const SimArgs &args, bool epoch, int total_warps, cudaStream_t s) {
+cudaError_t launch_sim(const SimArgs &args, int total_warps, cudaStream_t s) {
     int bps = 0, sms = 0, dev = 0;
     size_t smem = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    e = occupancy(args.B, args.n, epoch, dev, &bps, &sms, &smem);
+    e = occupancy(args.B, args.n, dev, &bps, &sms, &smem);
     if (e != cudaSuccess) return e;
     const int64_t n_tasks = args.n_inst * args.n_runs;
     int64_t blocks = total_warps / kSimWarpsPerBlock;
     const int64_t need = (n_tasks + kSimWarpsPerBlock - 1) / kSimWarpsPerBlock;
     if (blocks > need) blocks = need;
     if (blocks < 1) blocks = 1;
-    const void *k = pick_kernel(slots_per_lane(args.B), epoch);
+    const void *k = pick_kernel(slots_per_lane(args.B));
     SimArgs a = args;
     void *params[] = {&a, const_cast<int64_t *>(&n_tasks)};
     return cudaLaunchKernel(k, dim3((unsigned)blocks), dim3(kSimWarpsPerBlock * 32), params, smem, s);
