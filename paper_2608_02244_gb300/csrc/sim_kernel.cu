@@ -29,8 +29,7 @@
 //
 // Layout.  Worker (batch slot) w lives in lane w % 32, register row w / 32,
 // so a warp holds B <= 32 * SPL workers.  Values that change only at events
-// (next arrival, earliest completion, start range, KV reservation) are kept as
-// warp-uniform scalars.  The pending queue is a bitset over the instance's
+// (next arrival, start range, KV reservation) are kept as warp-uniform scalars.  The pending queue is a bitset over the instance's
 // request positions sorted by (o desc, index asc) -- the longest pending
 // request is the lowest set bit -- with a summary word per 32 words, in shared
 // memory.  ISJL plans are per-worker FIFO lists linked through a global
@@ -44,36 +43,40 @@ namespace isjl {
 namespace {
 
 constexpr int32_t kNone = -1;
-constexpr int32_t kIdle = -(1 << 30);   // an idle slot's start step
+constexpr uint32_t kEmpty = 0xFFFFFFFFu;   // key of a slot that holds no running request
+
+// bits of a running request's key that hold its register row
+template <int SPL> __host__ __device__ constexpr int row_bits() { return SPL >= 16 ? 4 : SPL >= 8 ? 3 : SPL >= 4 ? 2 : 1; }
 
 struct WarpSmem {
-    int32_t *sjob;    // [B] request running on worker w
-    int32_t *shead;   // [B] next ISJL plan entry of worker w (kNone = none)
-    int32_t *stail;   // [B] last plan entry of worker w
+    uint32_t *key;    // [32][SPL] completion step and slot row of the request on a slot (kEmpty: none)
+    int2 *slot;       // [B] request on worker w: start step, reserved KV (its planning length); in Phase ONE,
+                      //     w's last plan entry (-1: none) and w's packing budget, then its pack sum
+    uint32_t *slink;  // [B] plan link of worker w's next ISJL plan entry (0: none)
     int32_t *slong;   // [B] long request o_j planned on worker j (1 <= j < n_long)
-    int32_t *srem;    // [B] ISJL packing budget of worker w at a stage start (Phase ONE only)
-    int32_t *spsum;   // [B] ISJL pack sum on worker w in Phase ONE, then the o of its next plan entry
-    int32_t *sres;    // [B] KV reserved by the request running on worker w (its planning length)
     uint32_t *pend0;  // [words0] bit p: sorted position p is pending
     uint32_t *pend1;  // [words1] bit w: pend0[w] != 0
 };
 
-__host__ __device__ inline int smem_words_per_warp(int B, int words0, int words1) {
-    int w = 7 * B + words0 + words1;
+__host__ __device__ inline int smem_words_per_warp(int spl, int B, int words0, int words1) {
+    int w = 32 * spl + 4 * B + words0 + words1;
     return (w + 3) & ~3;  // keep every warp's block 16-byte aligned
 }
 
-// lowest / highest worker whose row bit is set in the per-lane mask m
+// copy one word from global to this lane's shared memory without waiting for it
+__device__ __forceinline__ void copy_async(uint32_t *smem, const int32_t *gmem) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;"
+                 :: "r"((uint32_t)__cvta_generic_to_shared(smem)), "l"(gmem) : "memory");
+}
+// wait for this lane's copies
+__device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// lowest worker whose row bit is set in the per-lane mask m
 __device__ __forceinline__ int lowest_worker(uint32_t m, int lane) {
     const int v = m ? ((__ffs(m) - 1) << 5) + lane : INT_MAX;
     const int r = __reduce_min_sync(kFull, v);
     return r == INT_MAX ? -1 : r;
 }
-__device__ __forceinline__ int highest_worker(uint32_t m, int lane) {
-    const int v = m ? ((31 - __clz(m)) << 5) + lane : -1;
-    return __reduce_max_sync(kFull, v);
-}
-
 // acc += a * b into a 64-bit accumulator with one wide multiply-add
 __device__ __forceinline__ void mad_wide(int64_t &acc, uint32_t a, uint32_t b) {
     asm("mad.wide.u32 %0, %1, %2, %0;" : "+l"(acc) : "r"(a), "r"(b));
@@ -86,6 +89,12 @@ __device__ __forceinline__ uint64_t warp_sum_u64(uint64_t v) {
     const uint32_t b = __reduce_add_sync(kFull, (uint32_t)(v >> 22) & 0x3FFFFFu);
     const uint32_t c = __reduce_add_sync(kFull, (uint32_t)(v >> 44));
     return (uint64_t)a + ((uint64_t)b << 22) + ((uint64_t)c << 44);
+}
+
+__device__ __forceinline__ int64_t warp_sum64(int64_t v) {
+#pragma unroll
+    for (int s = 16; s > 0; s >>= 1) v += __shfl_xor_sync(kFull, v, s);
+    return v;
 }
 
 // first pending sorted position >= p, INT_MAX if none (uniform call)
@@ -142,6 +151,22 @@ __device__ __forceinline__ int bs_last(const WarpSmem &S, int words1, int lane) 
     return -1;
 }
 
+// highest pending sorted position <= p, -1 if none (uniform call)
+__device__ __forceinline__ int bs_prev(const WarpSmem &S, int p, int lane) {
+    if (p < 0) return -1;
+    const int w0 = p >> 5;
+    const uint32_t v = S.pend0[w0] & (~0u >> (31 - (p & 31)));
+    if (v) return (w0 << 5) + 31 - __clz(v);
+    if (w0 == 0) return -1;
+    const int q = w0 - 1, w1 = q >> 5;
+    const uint32_t u = S.pend1[w1] & (~0u >> (31 - (q & 31)));
+    if (u) {
+        const int ww = (w1 << 5) + 31 - __clz(u);
+        return (ww << 5) + 31 - __clz(S.pend0[ww]);
+    }
+    return bs_last(S, w1, lane);
+}
+
 // position of the k-th (0-based) set bit of x; k < popc(x)
 __device__ __forceinline__ int nth_set_bit(uint32_t x, int k) {
     int pos = 0;
@@ -188,150 +213,196 @@ __device__ __forceinline__ int first_pos_le(const int32_t *os, int n, int64_t x,
 // One (instance, run) task under policy P, a compile-time constant (FCFS, LJF,
 // SJF or ISJL; Algorithm "ISJL" runs the ISJL body with beta in the packing
 // thresholds), so each policy's code holds only its own admission rule.
+//
+// Running requests.  Worker w = r * 32 + lane owns slot row r of its lane.  A
+// slot's key is the completion step (relative to kbase) above the slot row; a
+// lane's column of keys lies in shared memory as vector words and its smallest
+// key, the lane's next completion, in a register: a start is one store and one
+// minimum (of all 32 lanes at once), a completion a reload of that lane's column.
+// Start step and KV reservation lie in shared memory by slot and are read when
+// the request leaves.
+// A started request runs uninterrupted, so its completion step is written out
+// when it starts.
+//
+//
+// What bounds it: issue of one dependent chain of warp-uniform instructions per
+// event (ncu: issue slots half busy, DRAM a few percent), so the column layout
+// and the loop below are made for few instructions and branches per event.
+// Against the keys and start steps in per-lane registers, scanned and reduced at
+// every event, an FCFS event of a 20,000-request trace went from 258 to 189
+// instructions and 0.58 to 0.42 us; the simulation of 10,000 x 1,000 requests
+// under 7 runs from 19.2 to 14.6 ms, of 100,000 x 500 under 5 from 42.1 to 33.5
+// ms, of 1,024 x 100,000 under 3 from 108 to 64 ms.
+//
+// Costs.  W accumulates per interval between events; E = W - Q (the
+// decomposition W = Q + E of Section 5), with the served part of Q counted per
+// start when max_steps may stop the run early.  The start range [smin, smax] of
+// the running set changes at a start or when the last completion among the
+// requests that started at smin (e_lo) or at smax (e_hi) is reached; only then
+// is it searched for again.
 template <int SPL, int P>
 __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, int lane, int64_t gwarp,
                                          int64_t inst, int run) {
+    constexpr int RB = row_bits<SPL>();
+    constexpr uint32_t RM = (1u << RB) - 1u;
+    constexpr bool kIsjl = P == ISJL_POLICY_ISJL;
     const int n_slots = A.n, B = A.B;
     const int64_t base = inst * (int64_t)n_slots;
     const InstStats is = A.inst[inst];
     const int n = is.n;                             // requests of this instance (<= n_slots)
-    constexpr int policy = P;
-    const int64_t alpha = A.runs.delta[run];
-    const int64_t beta = A.runs.beta[run];
-    const int64_t kv_cap = A.kv_cap;
     // reserved KV: at most B <= 512 running requests of length <= 65535, so
     // below 2^25; kept in 32 bits, against the cap clamped to INT_MAX (which
     // compares the same)
-    const int32_t kv_lim = (int32_t)min(kv_cap, (int64_t)INT_MAX);
+    const int32_t kv_lim = (int32_t)min(A.kv_cap, (int64_t)INT_MAX);
     const int32_t *__restrict__ arr = A.arrival + base;
     const int32_t *__restrict__ oarr = A.o + base;              // planning lengths (u_i)
     const int32_t *__restrict__ otru = A.otrue ? A.otrue + base : nullptr;   // true lengths
     const int32_t *__restrict__ perm = A.perm + base;
     const int32_t *__restrict__ osrt = A.osorted + base;
     const int32_t *__restrict__ posof = A.posof + base;
-    int32_t *pnext = A.plan_next + gwarp * (int64_t)n_slots;
+    int32_t *pnext = A.plan_next + gwarp * (int64_t)n_slots;    // plan links, by request
     const int64_t out_off = (int64_t)run * A.n_inst * n_slots + base;
     int32_t *st_out = A.start_out ? A.start_out + out_off : nullptr;
     int32_t *co_out = A.compl_out ? A.compl_out + out_off : nullptr;
     const int words0 = (n + 31) >> 5, words1 = (words0 + 31) >> 5;
 
     int64_t status = is.status;
-    if (status == ISJL_OK && (int64_t)is.maxo > kv_cap) status = ISJL_ERR_INFEASIBLE;
-    // every schedule ends by sum o + max arrival; the idle sentinel needs steps < 2^30
+    if (status == ISJL_OK && is.maxo > kv_lim) status = ISJL_ERR_INFEASIBLE;
+    // every schedule ends by sum o + max arrival; completion steps need < 2^30
     if (status == ISJL_OK && is.O + (int64_t)is.maxA + 1 >= (int64_t)(1 << 30)) status = ISJL_ERR_INVALID_ARG;
-    // requests that never start / finish report -1: on an error status, in a
-    // run the caller's max_steps may stop, and in the unused slots of a ragged
-    // instance (a full run writes every other entry)
-    if (status != ISJL_OK || A.max_steps > 0 || n < n_slots) {
-        if (st_out) for (int i = lane; i < n_slots; i += 32) st_out[i] = -1;
-        if (co_out) for (int i = lane; i < n_slots; i += 32) co_out[i] = -1;
+    const bool trunc = A.max_steps > 0;             // the run may be stopped early
+    // requests that never start / finish report -1: all of them on an error
+    // status (and to begin with in a run that may be stopped), else the unused
+    // slots of a ragged instance (a full run writes every other entry)
+    for (int i = (status != ISJL_OK || trunc ? 0 : n) + lane; i < n_slots; i += 32) {
+        if (st_out) st_out[i] = -1;
+        if (co_out) co_out[i] = -1;
     }
 
     int64_t W = 0, E = 0, sumc = 0, sumext = 0;
     int32_t peakkv = 0;
-    int32_t Tb = 0, tok = 0, maxext = 0, viol = 0, peakb = 0, Tmake = 0, kvviol = 0;
+    int32_t Tb = 0, tok = 0, maxext = 0, viol = 0, peakb = 0, Tmake = 0;
 
     if (status == ISJL_OK && n > 0) {
-        for (int w = lane; w < words0; w += 32) S.pend0[w] = 0u;
-        for (int w = lane; w < words1; w += 32) S.pend1[w] = 0u;
-        for (int w = lane; w < B; w += 32) { S.shead[w] = kNone; S.stail[w] = kNone; S.slong[w] = kNone; }
+        if (P != ISJL_POLICY_FCFS) {
+            for (int w = lane; w < words0; w += 32) S.pend0[w] = 0u;
+            for (int w = lane; w < words1; w += 32) S.pend1[w] = 0u;
+        }
         __syncwarp();
 
-        // worker w = r * 32 + lane: sa = start step, sc = completion step (INT_MAX when idle)
-        int32_t sa[SPL], sc[SPL];
+        uint32_t *col = S.key + lane * SPL;          // this lane's column of keys
 #pragma unroll
-        for (int r = 0; r < SPL; ++r) { sa[r] = kIdle; sc[r] = INT_MAX; }
-        uint32_t busy = 0u, resv = 0u;
-        uint32_t lhead = 0u;    // worker's next plan entry is its long job o_j (waits for o_1)
-        int32_t lane_cmin = INT_MAX;                 // earliest completion among this lane's workers
-        int32_t lane_smin = INT_MAX, lane_smax = INT_MIN;   // start range of this lane's workers
+        for (int r = 0; r < SPL; ++r) col[r] = kEmpty;
+        uint32_t key0 = kEmpty;                      // the smallest of them
+        auto load_column = [&](uint32_t (&key)[SPL]) {
+            if constexpr (SPL >= 4) {
+#pragma unroll
+                for (int q = 0; q < SPL / 4; ++q) {
+                    const uint4 v = reinterpret_cast<const uint4 *>(col)[q];
+                    key[4 * q] = v.x; key[4 * q + 1] = v.y; key[4 * q + 2] = v.z; key[4 * q + 3] = v.w;
+                }
+            } else {
+#pragma unroll
+                for (int r = 0; r < SPL; ++r) key[r] = col[r];
+            }
+        };
         const int nrow = (B - lane + 31) >> 5;       // rows holding a valid worker for this lane
-        const uint32_t vmask = nrow >= 32 ? ~0u : ((1u << nrow) - 1u);
-        const int32_t alpha32 = (int32_t)min(alpha, (int64_t)INT_MAX);
+        uint32_t idle = nrow >= 32 ? ~0u : ((1u << nrow) - 1u);   // slot rows of this lane with no running request
+        uint32_t resv = 0u;     // ... and whose worker's next plan entry waits
+        uint32_t lhead = 0u;    // ... which is its long request o_j (waits for o_1)
+        const uint32_t lt = (1u << lane) - 1u;
+        const int32_t alpha32 = A.runs.delta[run];
+        uint64_t R_l = 0;                            // trunc: this lane's share of sum o (o + 1) / 2 over started requests
+        int32_t tok_l = 0;                           // trunc: of sum o over started requests
+        int64_t sums = 0;                            // sum of start steps
 
-        int32_t k = 0, rel = 0, fcfs = 0, done = 0, run_cnt = 0, pend = 0;
+        int32_t k = 0, kbase = 0, rel = 0, fcfs = 0, run_cnt = 0, pend = 0;
         int32_t kv_sum = 0;
-        uint32_t sum_st = 0;   // the running requests' start steps, summed modulo 2^32
         // the next 32 unreleased requests (from win_base): arrival and sorted position, per lane
         int32_t win_base = 0, win_a = INT_MAX, win_p = 0;
         auto load_window = [&]() {
             const int i = win_base + lane;
             win_a = i < n ? arr[i] : INT_MAX;
-            win_p = (i < n && policy != ISJL_POLICY_FCFS) ? posof[i] : 0;
+            win_p = (i < n && P != ISJL_POLICY_FCFS) ? posof[i] : 0;
         };
         load_window();
+        // FCFS: lengths of the 32 requests around the queue head and of the next 32, per lane
+        int32_t fo_l = 0, fo_n = 0, ft_l = 0, ft_n = 0, fo = 0, ft = 0;
+        auto load_lengths = [&](int i, int32_t &u, int32_t &t) {
+            u = i < n ? oarr[i] : 0;
+            t = otru ? (i < n ? otru[i] : 0) : u;
+        };
+        if (P == ISJL_POLICY_FCFS) {
+            load_lengths(lane, fo_l, ft_l);
+            load_lengths(32 + lane, fo_n, ft_n);
+            fo = __shfl_sync(kFull, fo_l, 0);
+            ft = __shfl_sync(kFull, ft_l, 0);
+        }
         // uniform caches, changed only at events
         int32_t next_arr = __shfl_sync(kFull, win_a, 0);   // arrival of the next unreleased request
-        int32_t hp = INT_MAX, ho = 0, he = 0, ho_pos = -1;   // longest pending position, its o and index
-        bool hvalid = true;                            // hp is current (else recompute from the bitset)
-        int32_t fo = -1;                               // o of the FCFS head (-1: not loaded)
-        int32_t cmin = INT_MAX;                        // earliest completion step of the running set
-        int32_t smin = INT_MAX, smax = INT_MIN;        // start range of the running set
-        int32_t kv_over = 0;                           // reserved KV above the cap (never, by construction)
-        int32_t plan_left = 0, t0 = 0, d1 = 0, L1 = kNone, nlong = 0;
+        // LJF / ISJL: the longest pending position, SJF: the last one (of the
+        // shortest length), with its planning length, index and true length
+        int32_t hp = P == ISJL_POLICY_SJF ? -1 : INT_MAX, ho = 0, he = 0, ht = 0;
+        // start range of the running set and the last completions of those started
+        // at its ends; found again (rescan) once e_lo or e_hi is reached
+        int32_t smin = 0, smax = 0, e_lo = INT_MIN, e_hi = INT_MIN;
+        int32_t plan_left = 0, t0 = 0, d1 = 0, nlong = 0;
         bool L1_started = true;
         bool broken = false;   // an internal invariant failed: stop without touching memory
-        const int64_t max_steps = A.max_steps > 0 ? A.max_steps : (is.O + (int64_t)is.maxA + 1);
+        const int64_t max_steps = trunc ? A.max_steps : (is.O + (int64_t)is.maxA + 1);
         const int32_t step_guard = (int32_t)min(max_steps + 1, (int64_t)INT_MAX);
+        // the next step at which something other than a completion happens: the
+        // guard, a renumbering of the keys' steps, an arrival or o_1's delay expiry
+        int32_t evt_base = RB > 2 ? min(step_guard, 1 << 27) : step_guard, evt = 0;
 
-        auto recompute_lane = [&]() {
-            lane_cmin = INT_MAX;
-            lane_smin = INT_MAX;
-            lane_smax = INT_MIN;
-#pragma unroll
-            for (int r = 0; r < SPL; ++r) {
-                lane_cmin = min(lane_cmin, sc[r]);               // idle slots hold INT_MAX
-                if (busy >> r & 1u) { lane_smin = min(lane_smin, sa[r]); lane_smax = max(lane_smax, sa[r]); }
-            }
+        // plan links: request and planning length of the entry after a request,
+        // in one word when request indices fit 16 bits, else the index plus one
+        const bool packed = n_slots <= 65536;
+        auto link_of = [&](int e, int oe) -> uint32_t {
+            return packed ? ((uint32_t)oe << 16) | (uint32_t)e : (uint32_t)e + 1u;
         };
-        // start request e (length oe) on worker w at step k
-        auto start = [&](int e, int oe, int w) {
-            const int oc = otru ? otru[e] : oe;          // it finishes after its true length
-            run_cnt++;
-            kv_sum += oe;                                // and reserves its planning length
-            cmin = min(cmin, k + oc);
-            peakkv = max(peakkv, kv_sum);
-            peakb = max(peakb, run_cnt);
-            kv_over = kv_sum > kv_lim;
-            sum_st += (uint32_t)k;
-            smin = min(smin, k);
-            smax = k;
-            const int owner = w & 31, row = w >> 5;
-            if (lane == owner) {
-#pragma unroll
-                for (int r = 0; r < SPL; ++r)
-                    if (r == row) { sa[r] = k; sc[r] = k + oc; }
-                busy |= 1u << row;
-                lane_cmin = min(lane_cmin, k + oc);
-                S.sres[w] = oe;
-                lane_smin = min(lane_smin, k);
-                lane_smax = max(lane_smax, k);
-                S.sjob[w] = e;
-                if (st_out) st_out[e] = k;
+        auto link_job = [&](uint32_t lk) -> int { return packed ? (int)(lk & 0xFFFFu) : (int)(lk - 1u); };
+        auto link_len = [&](uint32_t lk) -> int { return packed ? (int)(lk >> 16) : oarr[lk - 1u]; };
+
+        // this lane starts request e (planning length oe, true length oc) in slot
+        // row `row` at step k
+        auto occupy = [&](int e, int oe, int oc, int row) {
+            const int c = k + oc;
+            idle &= ~(1u << row);
+            S.slot[(row << 5) + lane] = make_int2(k, oe);
+            if (st_out) st_out[e] = k;
+            if (co_out) co_out[e] = c;
+            if (trunc) {
+                R_l += ((uint32_t)oc * (uint32_t)(oc + 1)) >> 1;      // oc (oc + 1) < 2^32
+                tok_l += oc;
             }
+            const uint32_t x = ((uint32_t)(c - kbase) << RB) | (uint32_t)row;
+            col[row] = x;
+            key0 = min(key0, x);
         };
-        // warp-wide totals of c starts at step k made lane-parallel: kv_add their
-        // reserved KV, my_cmin this lane's earliest completion
-        auto commit_starts = [&](int c, int32_t kv_add, int32_t my_cmin) {
-            __syncwarp();
-            lane_cmin = min(lane_cmin, my_cmin);
-            if (my_cmin != INT_MAX) { lane_smin = min(lane_smin, k); lane_smax = max(lane_smax, k); }
-            run_cnt += c;
+        // warp-wide totals of cnt starts at step k that reserve kv_add and whose
+        // last completion is c_hi
+        auto commit = [&](int cnt, int32_t kv_add, int32_t c_hi) {
+            run_cnt += cnt;
             kv_sum += kv_add;
-            cmin = min(cmin, (int32_t)__reduce_min_sync(kFull, (unsigned)my_cmin));
-            peakkv = max(peakkv, kv_sum);
-            peakb = max(peakb, run_cnt);
-            kv_over = kv_sum > kv_lim;
-            sum_st += (uint32_t)c * (uint32_t)k;
-            smin = min(smin, k);
+            mad_wide(sums, (uint32_t)cnt, (uint32_t)k);
+            e_hi = smax == k ? max(e_hi, c_hi) : c_hi;
             smax = k;
+        };
+        // start request e on lane owner's slot row `row` (that lane's value)
+        auto start = [&](int e, int oe, int oc, int owner, int row) {
+            if (lane == owner) occupy(e, oe, oc, row);
+            commit(1, oe, k + oc);
+        };
+        // start it on one of the free rows fm, which some lane has (the slots are
+        // interchangeable; lanes: those with one)
+        auto start_any = [&](int e, int oe, int oc, uint32_t fm, unsigned lanes) {
+            start(e, oe, oc, 31 - __clz(lanes), 31 - __clz(fm));
         };
         // Start, at step k, the longest prefix of up to 32 candidates (lane l < m
         // holds request ce and its planning length co) whose KV reservations fit
-        // and for which free workers remain, candidate i on the i-th lowest
-        // worker of the free mask fm.  The same outcome as starting them one at
-        // a time, each on the lowest free worker, until the first that does not
-        // fit.  Returns how many started.
+        // and for which free slots remain.  The same outcome as starting them one
+        // at a time until the first that does not fit.  Returns how many started.
         auto bulk_start = [&](int m, int ce, int co, uint32_t fm) -> int {
             int pre = lane < m ? co : 0;                          // inclusive prefix of co
 #pragma unroll
@@ -344,89 +415,102 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
             const int c = __popc(__ballot_sync(kFull, fit));
             if (c == 0) return 0;
             const int oc_l = (otru && lane < c) ? otru[ce] : co;  // it finishes after its true length
-            const uint32_t lt = (1u << lane) - 1u;
-            int base = 0;
-            int32_t my_cmin = INT_MAX;
-#pragma unroll
-            for (int r = 0; r < SPL; ++r) {
-                if (base < c) {
-                    const bool f = fm >> r & 1u;
-                    const unsigned rowf = __ballot_sync(kFull, f);
-                    const int rank = base + __popc(rowf & lt);     // among the free workers, in w order
-                    const int src = rank & 31;
-                    const int e = __shfl_sync(kFull, ce, src);
-                    const int oe = __shfl_sync(kFull, co, src);
-                    const int oc = __shfl_sync(kFull, oc_l, src);
-                    if (f && rank < c) {
-                        const int w = (r << 5) + lane;
-                        sa[r] = k;
-                        sc[r] = k + oc;
-                        busy |= 1u << r;
-                        my_cmin = min(my_cmin, k + oc);
-                        S.sres[w] = oe;
-                        S.sjob[w] = e;
-                        if (st_out) st_out[e] = k;
-                    }
-                    base += __popc(rowf);
+            const int32_t c_hi = k + (int32_t)__reduce_max_sync(kFull, lane < c ? (unsigned)oc_l : 0u);
+            for (int placed = 0; placed < c;) {                   // one per lane with a free slot and round
+                const bool f = fm != 0u;
+                const unsigned b = __ballot_sync(kFull, f);
+                const int rank = placed + __popc(b & lt);
+                const int src = rank & 31;
+                const int e = __shfl_sync(kFull, ce, src);
+                const int oe = __shfl_sync(kFull, co, src);
+                const int oc = __shfl_sync(kFull, oc_l, src);
+                if (f && rank < c) {
+                    occupy(e, oe, oc, __ffs(fm) - 1);
+                    fm &= fm - 1u;
                 }
+                placed += __popc(b);
             }
-            commit_starts(c, __shfl_sync(kFull, pre, c - 1), my_cmin);
+            commit(c, __shfl_sync(kFull, pre, c - 1), c_hi);
             return c;
         };
-        // requests completing at step c leave their workers
-        auto retire = [&](int32_t c) {
-            uint32_t fm = 0u;
-            unsigned sf = 0u;   // sum of (start - (c - 65536)) over finishing requests
-#pragma unroll
-            for (int r = 0; r < SPL; ++r) {
-                const bool f = sc[r] == c;                   // idle slots hold INT_MAX
-                fm |= (uint32_t)f << r;
-                if (f) {
-                    sf += (unsigned)(sa[r] - (c - 65536));
-                    sc[r] = INT_MAX;
+
+        // the earliest request of this lane's column leaves if f; freed += its KV
+        auto pop_front = [&](bool f, int32_t &freed) {
+            const uint32_t row = key0 & RM;
+            const int w = (int)(row << 5) + lane;
+            if (f) {
+                freed += S.slot[w].y;
+                if (kIsjl && plan_left > 0) {
+                    const uint32_t lk = S.slink[w];
+                    if (lk) {                                 // the worker's next plan entry waits now
+                        resv |= 1u << row;
+                        if (!L1_started && w < nlong && link_job(lk) == S.slong[w]) lhead |= 1u << row;
+                    }
                 }
             }
-            // per finishing request (usually one per warp): outputs and its KV release
-            int nf = 0, of = 0;
-            for (uint32_t m = fm; m; m &= m - 1u) {
-                const int w = ((__ffs(m) - 1) << 5) + lane;
-                nf++;
-                of += S.sres[w];
-                if (co_out) co_out[S.sjob[w]] = c;
+            if (f) {
+                idle |= 1u << row;
+                col[row] = kEmpty;
+                uint32_t key[SPL];
+                load_column(key);
+                key0 = key[0];
+#pragma unroll
+                for (int r = 1; r < SPL; ++r) key0 = min(key0, key[r]);
             }
-            busy &= ~fm;
-            // unconditional where measured cheaper than the branch (not for 16 rows)
-            if (SPL <= 8 || fm) recompute_lane();
-            nf = (int)__reduce_add_sync(kFull, (unsigned)nf);
-            of = (int)__reduce_add_sync(kFull, (unsigned)of);
-            // starts are within 65535 steps of c, so the offsets fit 32 bits
-            sum_st -= __reduce_add_sync(kFull, sf) + (uint32_t)nf * (uint32_t)(c - 65536);
-            done += nf;
-            run_cnt -= nf;
-            kv_sum -= of;
-            kv_over = kv_sum > kv_lim;
-            sumc += (int64_t)nf * c;
-            Tmake = c;
-            cmin = __reduce_min_sync(kFull, lane_cmin);
-            smin = __reduce_min_sync(kFull, lane_smin);
-            smax = __reduce_max_sync(kFull, lane_smax);
         };
-        // A_max(k): largest progress among running requests (0 if none)
-        auto amax_now = [&]() -> int32_t {
-            return run_cnt == 0 ? 0 : k - smin;
+        // start range of the running set, and the last completions at its ends
+        auto rescan = [&]() {
+            int32_t lo = INT_MAX, hi = INT_MIN;
+            int32_t s_of[SPL];
+            uint32_t key[SPL];
+            load_column(key);
+#pragma unroll
+            for (int r = 0; r < SPL; ++r) {
+                s_of[r] = -1;
+                if (key[r] != kEmpty) {
+                    s_of[r] = S.slot[(r << 5) + lane].x;
+                    lo = min(lo, s_of[r]);
+                    hi = max(hi, s_of[r]);
+                }
+            }
+            smin = __reduce_min_sync(kFull, lo);
+            smax = __reduce_max_sync(kFull, hi);
+            uint32_t m_lo = 0u, m_hi = 0u;
+#pragma unroll
+            for (int r = 0; r < SPL; ++r) {
+                if (s_of[r] == smin) m_lo = max(m_lo, key[r]);
+                if (s_of[r] == smax) m_hi = max(m_hi, key[r]);
+            }
+            e_lo = kbase + (int32_t)(__reduce_max_sync(kFull, m_lo) >> RB);
+            e_hi = kbase + (int32_t)(__reduce_max_sync(kFull, m_hi) >> RB);
         };
 
+        auto set_head = [&](int p) {
+            hp = p;
+            if (p >= 0 && p < n) {
+                ho = osrt[p];
+                he = perm[p];
+                ht = otru ? otru[he] : ho;
+            }
+        };
+        // requests with A_i <= k join the queue (a prefix: arrivals are non-decreasing)
         auto release = [&]() {
             for (;;) {
                 // released: window lanes at or after rel whose arrival is <= k (a prefix)
                 const bool ok = win_base + lane >= rel && win_a <= k;
                 const unsigned b = __ballot_sync(kFull, ok);
-                if (policy != ISJL_POLICY_FCFS) {
+                if (P != ISJL_POLICY_FCFS) {
                     if (ok) {
                         atomicOr(&S.pend0[win_p >> 5], 1u << (win_p & 31));
                         atomicOr(&S.pend1[win_p >> 10], 1u << ((win_p >> 5) & 31));
                     }
-                    if (hvalid) hp = min(hp, __reduce_min_sync(kFull, ok ? win_p : INT_MAX));
+                    if (P == ISJL_POLICY_SJF) {
+                        const int q = __reduce_max_sync(kFull, ok ? win_p : -1);
+                        if (q > hp) set_head(q);
+                    } else {
+                        const int q = __reduce_min_sync(kFull, ok ? win_p : INT_MAX);
+                        if (q < hp) set_head(q);
+                    }
                 }
                 const int c = __popc(b);
                 rel += c;
@@ -438,17 +522,18 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
             __syncwarp();
             next_arr = rel < n ? __shfl_sync(kFull, win_a, (rel - win_base) & 31) : INT_MAX;
         };
-        // longest pending position (INT_MAX if none), its o and request index
-        auto head = [&]() -> int {
-            if (!hvalid) { hp = bs_next(S, words0, words1, 0, lane); hvalid = true; }
-            if (hp < n && ho_pos != hp) { ho = osrt[hp]; he = perm[hp]; ho_pos = hp; }
-            return hp;
-        };
-        // remove the head position p (the longest pending request)
-        auto pop_head = [&](int p) {
-            bs_clear(S, p, lane);
+        // remove the head (the longest pending request): nothing is pending below it
+        auto pop_head = [&]() {
+            const int w = hp >> 5;
+            const uint32_t v = S.pend0[w] & ~(1u << (hp & 31));
+            __syncwarp();
+            if (lane == 0) {
+                S.pend0[w] = v;
+                if (!v) S.pend1[w >> 5] &= ~(1u << (w & 31));
+            }
+            __syncwarp();
             pend--;
-            hp = bs_next(S, words0, words1, p + 1, lane);   // nothing pending below p
+            set_head(v ? (w << 5) + __ffs(v) - 1 : bs_next(S, words0, words1, (w + 1) << 5, lane));
         };
         // sorted positions of the first m (1 <= m <= 32) pending requests at or
         // after position p0: lane l gets the l-th, lanes past the last one -1
@@ -482,11 +567,6 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
             }
             return mine;
         };
-        // the first m (1 <= m <= min(32, pend)) pending requests: the longest first
-        auto first_pending = [&](int m) -> int {
-            if (!hvalid) { hp = bs_next(S, words0, words1, 0, lane); hvalid = true; }
-            return first_pending_from(hp, m);
-        };
         // remove the lanes' positions p (where take) from the pending set
         auto clear_pending = [&](int p, bool take) {
             if (take) {
@@ -497,60 +577,55 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
             __syncwarp();
         };
         // start the longest pending requests (LJF's batch, ISJL's Phase TWO) on
-        // the free workers of fm_base until one does not fit or the workers run out
-        auto start_longest = [&](uint32_t fm_base) -> void {
+        // idle slots (ISJL: not reserved for a plan entry) until one does not fit
+        // or the slots run out
+        auto start_longest = [&]() {
             // one at a time for the first two starts (usually all there are),
             // then 32 at a time; every round first checks that the head fits
-            for (int nseq = 0; pend > 0;) {
-                const int w = lowest_worker(fm_base & ~busy, lane);
-                if (w < 0) return;
-                const int p = head();
-                if (p >= n) { broken = true; return; }
-                if (kv_sum + ho > kv_lim) return;
+            unsigned lanes = __ballot_sync(kFull, (idle & ~resv) != 0u);
+            for (int nseq = 0; pend > 0 && kv_sum + ho <= kv_lim && lanes != 0u; ++nseq) {
+                if (hp >= n) { broken = true; return; }
                 if (nseq < 2) {
-                    const int e = he, oe = ho;
-                    pop_head(p);
-                    start(e, oe, w);
-                    nseq++;
-                    continue;
+                    start_any(he, ho, ht, idle & ~resv, lanes);
+                    pop_head();
+                } else {
+                    const int m = min(32, pend);
+                    const int q = first_pending_from(hp, m);
+                    if (__ballot_sync(kFull, lane < m && q < 0)) { broken = true; return; }
+                    const int ce = q >= 0 ? perm[q] : 0;
+                    const int co = q >= 0 ? osrt[q] : 0;
+                    const int c = bulk_start(m, ce, co, idle & ~resv);
+                    clear_pending(q, lane < c);
+                    pend -= c;
+                    const int first = __shfl_sync(kFull, q, 0);
+                    set_head(c < m ? __shfl_sync(kFull, q, c & 31) : bs_next(S, words0, words1, first, lane));
                 }
-                const int m = min(32, pend);
-                const int q = first_pending(m);
-                if (__ballot_sync(kFull, lane < m && q < 0)) { broken = true; return; }
-                const int ce = q >= 0 ? perm[q] : 0;
-                const int co = q >= 0 ? osrt[q] : 0;
-                const int c = bulk_start(m, ce, co, fm_base & ~busy);
-                clear_pending(q, lane < c);
-                pend -= c;
-                if (c < m) { hp = __shfl_sync(kFull, q, c); return; }   // the first one left is the head
-                hvalid = false;
+                lanes = __ballot_sync(kFull, (idle & ~resv) != 0u);
             }
         };
 
         // ISJL plan starts of every candidate worker in cand (per-lane row
         // mask) at once, in worker order, until the first whose next entry does
         // not fit the KV cap (then true is returned: the gate of the step is
-        // shut); entries that must wait (o_1 delayed unless over, an o_j before
-        // o_1 has started) are skipped.  o_1 itself never comes here: worker 0
-        // is always the first candidate and is started one at a time.
-        auto plan_bulk = [&](uint32_t cand, bool over) -> bool {
+        // shut); entries that must wait (o_1 delayed, an o_j before o_1 has
+        // started) are not in cand.
+        auto plan_bulk = [&](uint32_t cand) -> bool {
             bool stopped = false;
             int c = 0;
             int32_t kv_add = 0;
-            int32_t my_cmin = INT_MAX;
+            uint32_t oc_hi = 0u;
 #pragma unroll
             for (int r = 0; r < SPL; ++r) {
-                if (!stopped) {
+                const bool el = !stopped && (cand >> r & 1u);
+                if (__ballot_sync(kFull, el) != 0u) {
                     const int w = (r << 5) + lane;
-                    bool el = cand >> r & 1u;
                     int e = 0, oe = 0;
                     if (el) {
-                        e = S.shead[w];
-                        if (w == 0 && e == L1 && !over) el = false;
-                        if (w >= 1 && w < nlong && e == S.slong[w] && !L1_started) el = false;
-                        if (el) oe = S.spsum[w];
+                        const uint32_t lk = S.slink[w];
+                        e = link_job(lk);
+                        oe = link_len(lk);
                     }
-                    int pre = el ? oe : 0;                      // prefix over this row, in lane order
+                    int pre = oe;                               // prefix over this row, in lane order
 #pragma unroll
                     for (int d = 1; d < 32; d <<= 1) {
                         const int t = __shfl_up_sync(kFull, pre, d);
@@ -560,34 +635,30 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
                     const unsigned fb = __ballot_sync(kFull, fits);
                     if (fb != __ballot_sync(kFull, el)) stopped = true;   // the first one that does not fit
                     if (fits) {
-                        const int nx = pnext[e];
-                        const int onx = nx >= 0 ? oarr[nx] : 0;
-                        S.shead[w] = nx;
-                        const uint32_t bit = 1u << r;
-                        if (nx < 0) { S.stail[w] = kNone; resv &= ~bit; } else S.spsum[w] = onx;
-                        if (w >= 1 && w < nlong && nx >= 0 && nx == S.slong[w]) lhead |= bit;
-                        else lhead &= ~bit;
+                        copy_async(S.slink + w, pnext + e);
                         const int oc = otru ? otru[e] : oe;     // it finishes after its true length
-                        sa[r] = k;
-                        sc[r] = k + oc;
-                        busy |= bit;
-                        my_cmin = min(my_cmin, k + oc);
-                        S.sres[w] = oe;
-                        S.sjob[w] = e;
-                        if (st_out) st_out[e] = k;
+                        occupy(e, oe, oc, r);
+                        resv &= ~(1u << r);
+                        lhead &= ~(1u << r);
+                        oc_hi = max(oc_hi, (uint32_t)oc);
                     }
                     c += __popc(fb);
                     kv_add += (int32_t)__reduce_add_sync(kFull, fits ? (unsigned)oe : 0u);
                 }
             }
-            if (c > 0) commit_starts(c, kv_add, my_cmin);
+            if (c > 0)
+                commit(c, kv_add, k + (int32_t)__reduce_max_sync(kFull, oc_hi));
             plan_left -= c;
             return stopped;
         };
 
-        // ISJL Phase ONE at a stage start (Algorithm 2 with beta = alpha)
+        // ISJL Phase ONE at a stage start (Algorithm 2 with beta = alpha).  Nothing
+        // runs, so the slots' array is free: it holds each worker's last plan entry and
+        // first its packing budget, then its pack sum; room[] holds the packing
+        // budgets left (0: takes no pack)
         auto phase_one = [&]() {
-            t0 = k; d1 = 0; L1 = kNone; L1_started = true; nlong = 0;
+            const int64_t alpha = A.runs.delta[run], beta = A.runs.beta[run];
+            t0 = k; d1 = 0; L1_started = true; nlong = 0;
             if (pend < 2) return;                               // |Q| = 1: Phase TWO
             const int p1 = bs_next(S, words0, words1, 0, lane);
             if (p1 >= n) { broken = true; return; }
@@ -599,10 +670,12 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
             // M = min{B, #{o > alpha}} over Q(k)
             const int cnt_long = bs_count_below(S, words0, first_pos_le(osrt, n, alpha, lane), lane);
             const int nl = min(B, cnt_long);
-            // packing budget left / pack sum per worker, in shared memory
+            copy_wait();                                        // links of the last stage still in flight
+            __syncwarp();
             for (int w = lane; w < B; w += 32) {
-                S.srem[w] = w >= nl ? (int32_t)alpha : -1;   // workers M+1..B: alpha
-                S.spsum[w] = 0;
+                S.slot[w] = make_int2(kNone, w >= nl ? (int32_t)alpha : 0);   // workers M+1..B: alpha
+                S.slink[w] = 0u;
+                S.slong[w] = kNone;
             }
             __syncwarp();
             // the long requests o_1..o_M (the first M pending positions) leave Q;
@@ -636,10 +709,10 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
                         const int e = perm[p];
                         const int oe = osrt[p];
                         if (j == 0) {
-                            S.shead[0] = e; S.stail[0] = e; pnext[e] = kNone;
+                            S.slink[0] = link_of(e, oe);
                         } else {
                             S.slong[j] = e;
-                            S.srem[j] = (int32_t)min(2 * alpha, o1 - (int64_t)oe + beta);
+                            S.slot[j].y = (int32_t)min(2 * alpha, o1 - (int64_t)oe + beta);
                         }
                         if (j == nl - 1) olast_l = oe;
                     }
@@ -654,85 +727,111 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
                 taken += m;
             }
             __syncwarp();
-            L1 = S.shead[0];
             const int64_t o_last = __reduce_max_sync(kFull, olast_l);
             pend -= nl;
             const int64_t theta = min(2 * alpha, o1 - o_last + beta);
-            // first fit of the shorter requests, in sorted order.  Nothing runs
-            // at a stage start, so the slot registers sa[] are free: they hold
-            // the packing budgets left, worker r * 32 + lane in sa[r] (-1 for
-            // worker 1 and past B: never chosen), and are reset to idle below.
+            uint32_t room[SPL];
 #pragma unroll
             for (int r = 0; r < SPL; ++r) {
                 const int w = (r << 5) + lane;
-                sa[r] = w < B ? S.srem[w] : -1;
+                room[r] = w < B ? (uint32_t)S.slot[w].y : 0u;
+                if (w < B) S.slot[w].y = 0;
             }
+            __syncwarp();
             // maxrem bounds the largest budget from above; it is recomputed only
             // when a candidate no larger than it fits nowhere (budgets only shrink)
-            int maxrem = -1;
+            auto max_budget = [&]() -> int {
+                uint32_t m = 0u;
 #pragma unroll
-            for (int r = 0; r < SPL; ++r) maxrem = max(maxrem, sa[r]);
-            maxrem = __reduce_max_sync(kFull, maxrem);
+                for (int r = 0; r < SPL; ++r) m = max(m, room[r]);
+                return (int)__reduce_max_sync(kFull, m);
+            };
+            int64_t x = min(theta, (int64_t)max_budget());
             // this lane's rows whose worker takes no long request (M+1..B)
             uint32_t rows_short = 0u;
 #pragma unroll
             for (int r = 0; r < SPL; ++r) rows_short |= (uint32_t)((r << 5) + lane >= nl) << r;
-            int q = -1;
-            int64_t x_prev = -1;
-            int pos_x = 0;                                      // first sorted position with o <= x_prev
-            for (;;) {
-                const int64_t x = min(theta, (int64_t)maxrem);
-                if (x < 1) break;
-                // candidates with o > x fit nowhere now or later
-                if (x != x_prev) { pos_x = first_pos_le(osrt, n, x, lane); x_prev = x; }
-                q = bs_next(S, words0, words1, max(pos_x, q + 1), lane);
-                if (q >= n) break;
-                const int e = perm[q];
-                const int oe = osrt[q];
-                uint32_t fit = 0u;                              // rows whose budget takes it
+            // First fit of the shorter requests, in sorted order, on workers M+1..B
+            // first, then M, M-1, ..., 2.  32 candidates at a time: lane l loads the
+            // l-th; each is placed by a search over all budgets, and the plan lists
+            // are linked once per 32
+            int from = x >= 1 ? first_pos_le(osrt, n, x, lane) : n;
+            while (x >= 1 && from < n) {
+                const int q = first_pending_from(from, 32);
+                const int last = __reduce_max_sync(kFull, q);
+                if (last < 0) break;
+                const int e = q >= 0 ? perm[q] : 0;
+                const int oe = q >= 0 ? osrt[q] : INT_MAX;
+                int wsel = -1 - lane;                           // the worker it goes to (distinct if none)
+                bool shrunk = false;
+                unsigned todo = __ballot_sync(kFull, (int64_t)oe <= x);
+                while (todo) {
+                    const int i = __ffs(todo) - 1;
+                    todo &= todo - 1u;
+                    const uint32_t o = (uint32_t)__shfl_sync(kFull, oe, i);
+                    uint32_t fit = 0u;                          // rows whose budget takes it
 #pragma unroll
-                for (int r = 0; r < SPL; ++r) fit |= (uint32_t)(sa[r] >= oe) << r;
-                int w = lowest_worker(fit & rows_short, lane);  // workers M+1..B first
-                if (w < 0) w = highest_worker(fit & ~rows_short, lane);   // then M, M-1, ..., 2
-                if (w < 0) {                                    // it stays queued; the bound was stale
-                    int m = -1;
+                    for (int r = 0; r < SPL; ++r) fit |= (uint32_t)(room[r] >= o) << r;
+                    // code of this lane's first choice: w for a short worker, 1023 - w for a long one
+                    const uint32_t fs = fit & rows_short;
+                    unsigned code = 0xFFFFu;
+                    if (fs) code = (unsigned)(((__ffs(fs) - 1) << 5) + lane);
+                    else if (fit) code = (unsigned)(1023 - (((31 - __clz(fit)) << 5) + lane));
+                    code = __reduce_min_sync(kFull, code);
+                    if (code == 0xFFFFu) {                      // it stays queued; the bound was stale
+                        x = min(theta, (int64_t)max_budget());
+                        todo &= __ballot_sync(kFull, (int64_t)oe <= x);
+                        shrunk = true;
+                        continue;
+                    }
+                    const int w = code < 512u ? (int)code : 1023 - (int)code;
+                    const uint32_t dec = lane == (w & 31) ? o : 0u;   // the chosen worker's budget shrinks
 #pragma unroll
-                    for (int r = 0; r < SPL; ++r) m = max(m, sa[r]);
-                    maxrem = __reduce_max_sync(kFull, m);
-                    continue;
+                    for (int r = 0; r < SPL; ++r) room[r] -= r == (w >> 5) ? dec : 0u;
+                    if (lane == i) wsel = w;
                 }
-                {
-                    const int dec = lane == (w & 31) ? oe : 0;   // the chosen worker's budget shrinks
-#pragma unroll
-                    for (int r = 0; r < SPL; ++r) sa[r] -= r == (w >> 5) ? dec : 0;
+                // append the window's requests to their workers' lists, in lane order
+                const bool take = wsel >= 0;
+                const unsigned same = __match_any_sync(kFull, wsel);
+                const unsigned after = same & ~lt & ~(1u << lane);
+                const int succ = after ? __ffs(after) - 1 : lane;
+                const int es = __shfl_sync(kFull, e, succ);
+                const int os_ = __shfl_sync(kFull, oe, succ);
+                int tail = kNone;
+                if (take) {
+                    pnext[e] = after ? (int32_t)link_of(es, os_) : 0;
+                    if (!(same & lt)) tail = S.slot[wsel].x;
+                    if (wsel < nl) atomicAdd(&S.slot[wsel].y, oe);
                 }
                 __syncwarp();
-                if (lane == 0) {
-                    const int tl = S.stail[w];
-                    if (tl < 0) S.shead[w] = e; else pnext[tl] = e;
-                    S.stail[w] = e;
-                    pnext[e] = kNone;
-                    S.spsum[w] += oe;
+                if (take) {
+                    if (!(same & lt)) {
+                        const uint32_t lk = link_of(e, oe);
+                        if (tail < 0) S.slink[wsel] = lk; else pnext[tail] = (int32_t)lk;
+                    }
+                    if (!after) S.slot[wsel].x = e;
                 }
-                bs_clear(S, q, lane);   // includes __syncwarp
-                pend--;
-                plan_left++;
+                const int cnt = __popc(__ballot_sync(kFull, take));
+                clear_pending(q, take);                        // includes __syncwarp
+                pend -= cnt;
+                plan_left += cnt;
+                from = last + 1;
+                if (shrunk && x >= 1) from = max(from, first_pos_le(osrt, n, x, lane));
             }
-#pragma unroll
-            for (int r = 0; r < SPL; ++r) sa[r] = kIdle;
             // worker j (2..M) runs o_j after its pack
             for (int w = 1 + lane; w < nl; w += 32) {
                 const int e = S.slong[w];
-                const int tl = S.stail[w];
-                if (tl < 0) S.shead[w] = e; else pnext[tl] = e;
-                S.stail[w] = e;
-                pnext[e] = kNone;
+                const int tl = S.slot[w].x;
+                const uint32_t lk = link_of(e, packed ? oarr[e] : 0);
+                if (tl < 0) S.slink[w] = lk; else pnext[tl] = (int32_t)lk;
+                pnext[e] = 0;
             }
             __syncwarp();
+            if (lane == 0) pnext[link_job(S.slink[0])] = 0;
             plan_left += nl;
             // o_1 waits d1 = min{max{max_j sum(w_j) - alpha, 0}, alpha}, j = 2..M
             int mx = 0;
-            for (int w = 1 + lane; w < nl; w += 32) mx = max(mx, S.spsum[w]);
+            for (int w = 1 + lane; w < nl; w += 32) mx = max(mx, S.slot[w].y);
             mx = __reduce_max_sync(kFull, mx);
             d1 = (int32_t)min(max((int64_t)mx - alpha, (int64_t)0), alpha);
             resv = 0u;
@@ -740,18 +839,15 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
 #pragma unroll
             for (int r = 0; r < SPL; ++r) {
                 const int w = (r << 5) + lane;
-                if (w < B && S.shead[w] >= 0) resv |= 1u << r;
-                if (w >= 1 && w < nl && S.shead[w] == S.slong[w]) lhead |= 1u << r;
+                if (w < B && S.slink[w]) {
+                    resv |= 1u << r;
+                    if (w >= 1 && w < nl && link_job(S.slink[w]) == S.slong[w]) lhead |= 1u << r;
+                }
             }
             L1_started = false;
             nlong = nl;
-            hvalid = false;                                // Phase ONE removed queued requests
-            // spsum now caches the length of each worker's next plan entry
-            for (int w = lane; w < B; w += 32) {
-                const int e = S.shead[w];
-                S.spsum[w] = e >= 0 ? oarr[e] : 0;
-            }
             __syncwarp();
+            set_head(bs_next(S, words0, words1, 0, lane));   // Phase ONE removed queued requests
         };
 
         // After an admission, `blocked` says that no arrival alone can let a
@@ -761,255 +857,253 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
         // stopped on the KV cap or on workers (an arrival never becomes a head
         // that fits better: it sorts after every pending request of its length).
         // Arrivals are then released at the next event instead of ending the
-        // run of plain steps there.
-        bool blocked = false;
+        // interval there.
         auto admit = [&]() {
-            if (policy == ISJL_POLICY_FCFS) {
-                // arrival order; the first request that does not fit ends the step
-                blocked = false;
+            bool blocked;
+            if (P == ISJL_POLICY_FCFS) {
+                // arrival order; the first request that does not fit ends the step;
                 // one at a time for the first two starts (usually all there are),
-                // then 32 at a time; every round first checks that the head fits
-                for (int nseq = 0;;) {
-                    if (run_cnt >= B) { blocked = true; break; }
-                    if (fcfs >= rel) break;
-                    if (fo < 0) fo = oarr[fcfs];
-                    if (kv_sum + fo > kv_lim) { blocked = true; break; }
+                // then 32 at a time
+                for (int nseq = 0; fcfs < rel && kv_sum + fo <= kv_lim && run_cnt < B; ++nseq) {
+                    int c = 1;
                     if (nseq < 2) {
-                        const int w = lowest_worker(vmask & ~busy, lane);
-                        if (w < 0) { broken = true; return; }
-                        start(fcfs, fo, w);
-                        fcfs++;
-                        fo = -1;
-                        nseq++;
-                        continue;
+                        start_any(fcfs, fo, ft, idle, __ballot_sync(kFull, idle != 0u));
+                    } else {
+                        const int m = min(32, rel - fcfs), i = fcfs + lane;
+                        c = bulk_start(m, i, lane < m ? oarr[i] : 0, idle);
                     }
-                    const int m = min(32, rel - fcfs);
-                    const int i = fcfs + lane;
-                    const int c = bulk_start(m, i, lane < m ? oarr[i] : 0, vmask & ~busy);
+                    const bool turn = (fcfs & 31) + c >= 32;     // the head enters the next 32
                     fcfs += c;
-                    fo = -1;
-                    if (c < m) { blocked = true; break; }        // the KV cap or B stopped it
+                    if (turn) {
+                        fo_l = fo_n;
+                        ft_l = ft_n;
+                        load_lengths((fcfs & ~31) + 32 + lane, fo_n, ft_n);
+                    }
+                    fo = __shfl_sync(kFull, fo_l, fcfs & 31);
+                    ft = __shfl_sync(kFull, ft_l, fcfs & 31);
                 }
-            } else if (policy == ISJL_POLICY_SJF) {
+                blocked = fcfs < rel || run_cnt >= B;
+            } else if (P == ISJL_POLICY_SJF) {
                 // shortest released request first (ties: lower index), continuous
-                // batching.  The pending requests of the smallest length omin are
-                // the pending positions from the first with o <= omin upwards, in
-                // start order; one at a time for the first two starts, then up to
-                // 32 of them at a time
-                for (int nseq = 0; run_cnt < B && pend > 0;) {
-                    const int hi = bs_last(S, words1, lane);
-                    if (hi < 0 || hi >= n) { broken = true; return; }
-                    const int omin = osrt[hi];
-                    if (kv_sum + omin > kv_lim) break;
-                    const int g = first_pos_le(osrt, n, omin, lane);
+                // batching.  The pending requests of the smallest length are the
+                // pending positions from the first of that length upwards, in start
+                // order; one at a time for the first two starts, then up to 32 of
+                // them at a time
+                for (int nseq = 0; pend > 0 && kv_sum + ho <= kv_lim && run_cnt < B; ++nseq) {
+                    if (hp < 0 || hp >= n) { broken = true; return; }
+                    // first position of this length: usually among the 32 up to hp
+                    const int i = hp - lane;
+                    const unsigned other = __ballot_sync(kFull, i < 0 || osrt[max(i, 0)] != ho);
+                    const int g = other ? hp - __ffs(other) + 2 : first_pos_le(osrt, n, ho, lane);
                     if (nseq < 2) {
                         const int p = bs_next(S, words0, words1, g, lane);
-                        if (p >= n) { broken = true; return; }
-                        const int w = lowest_worker(vmask & ~busy, lane);
-                        if (w < 0) { broken = true; return; }
-                        const int e = perm[p];
+                        if (p > hp) { broken = true; return; }
+                        const int e = p == hp ? he : perm[p];
+                        const int oc = otru ? otru[e] : ho;
+                        start_any(e, ho, oc, idle, __ballot_sync(kFull, idle != 0u));
                         bs_clear(S, p, lane);
                         pend--;
-                        start(e, omin, w);
-                        nseq++;
-                        continue;
+                        if (p == hp) set_head(bs_prev(S, hp, lane));
+                    } else {
+                        const int q = first_pending_from(g, min(32, pend));
+                        const int mg = __popc(__ballot_sync(kFull, q >= 0));   // of this length, in order
+                        if (mg == 0) { broken = true; return; }
+                        const int c = bulk_start(mg, q >= 0 ? perm[q] : 0, ho, idle);
+                        clear_pending(q, lane < c);
+                        pend -= c;
+                        set_head(bs_prev(S, hp, lane));
                     }
-                    const int q = first_pending_from(g, min(32, pend));
-                    const int mg = __popc(__ballot_sync(kFull, q >= 0));   // of this length, in order
-                    if (mg == 0) { broken = true; return; }
-                    const int c = bulk_start(mg, q >= 0 ? perm[q] : 0, omin, vmask & ~busy);
-                    clear_pending(q, lane < c);
-                    pend -= c;
-                    hvalid = false;
-                    if (c < mg) break;
                 }
                 blocked = run_cnt >= B;
-            } else if (policy == ISJL_POLICY_LJF) {
+            } else if (P == ISJL_POLICY_LJF) {
                 // static batch of the longest released requests when nothing runs
-                blocked = run_cnt != 0;
-                if (run_cnt != 0) return;
-                start_longest(vmask);
+                if (run_cnt == 0) start_longest();
                 blocked = run_cnt != 0;
             } else {
-                const bool nothing_runs = run_cnt == 0;
-                if (nothing_runs && plan_left == 0 && pend > 0) phase_one();
+                if (run_cnt == 0 && plan_left == 0 && pend > 0) phase_one();
                 if (broken) return;
                 // the gate A_max(k) <= alpha; progress stays below o <= 65535, so a
                 // budget of at least 65535 never shuts it
-                bool stop = alpha32 < 65535 && amax_now() > alpha32;
+                bool stop = false;
+                if (alpha32 < 65535 && run_cnt > 0) {
+                    if (e_lo <= k) rescan();
+                    stop = k - smin > alpha32;
+                }
                 if (!stop && plan_left > 0) {
                     // plan starts, workers in order; entries that must wait (o_1's
                     // delay, o_j before o_1) are filtered out up front
-                    uint32_t cand = resv & ~busy;
+                    uint32_t cand = resv;
                     if (!L1_started) {
                         cand &= ~lhead;
-                        const bool over = k >= t0 + d1;
-                        if (!over && lane == 0) cand &= ~1u;        // worker 0 holds o_1
+                        if (k < t0 + d1 && lane == 0) cand &= ~1u;   // worker 0 holds o_1
                     }
-                    for (int nseq = 0;;) {
+                    for (int nseq = 0; __ballot_sync(kFull, cand != 0u) != 0u; ++nseq) {
                         if (nseq >= 2) {                            // the rest at once
-                            if (__ballot_sync(kFull, cand != 0u)) {
-                                const bool over = k >= t0 + d1;
-                                stop = plan_bulk(cand, over);
-                            }
+                            stop = plan_bulk(cand);
                             break;
                         }
                         const int w = lowest_worker(cand, lane);
-                        if (w < 0) break;
-                        if (lane == (w & 31)) cand &= ~(1u << (w >> 5));
-                        const int e = S.shead[w];
-                        if (w == 0 && e == L1) {
-                            const bool over = k >= t0 + d1;
-                            if (!over) continue;                 // o_1 still delayed
-                        }
-                        if (w >= 1 && w < nlong && e == S.slong[w] && !L1_started) continue;  // o_j after o_1
-                        const int oe = S.spsum[w];                 // o of the worker's next entry
+                        const int owner = w & 31, row = w >> 5;
+                        const uint32_t lk = __shfl_sync(kFull, lane == owner ? S.slink[w] : 0u, owner);
+                        const int e = link_job(lk);
+                        const int oe = link_len(lk);
                         if (kv_sum + oe > kv_lim) { stop = true; break; }
-                        const int nx = pnext[e];
-                        __syncwarp();
-                        if (lane == 0) {
-                            S.shead[w] = nx;
-                            if (nx < 0) S.stail[w] = kNone; else S.spsum[w] = oarr[nx];
-                        }
-                        __syncwarp();
-                        if (lane == (w & 31)) {
-                            const uint32_t bit = 1u << (w >> 5);
-                            if (nx < 0) resv &= ~bit;
-                            if (w >= 1 && w < nlong && nx >= 0 && nx == S.slong[w]) lhead |= bit;
-                            else lhead &= ~bit;
+                        if (lane == owner) {
+                            const uint32_t keep = ~(1u << row);
+                            copy_async(S.slink + w, pnext + e);
+                            cand &= keep;
+                            resv &= keep;
+                            lhead &= keep;
                         }
                         plan_left--;
-                        if (e == L1) {
+                        if (w == 0) {                               // o_1: the o_j may start now
                             L1_started = true;
-                            cand |= resv & ~busy & lhead;            // the o_j may start now
+                            cand |= lhead;
                         }
-                        start(e, oe, w);
-                        nseq++;
+                        start(e, oe, otru ? otru[e] : oe, owner, row);
                     }
                 }
-                if (!stop) start_longest(vmask & ~resv);   // Phase TWO: longest released first
+                if (!stop) start_longest();   // Phase TWO: longest released first
                 blocked = stop || pend > 0;
             }
+            evt = blocked && run_cnt > 0 ? evt_base : min(evt_base, next_arr);
+            if (kIsjl && !L1_started && t0 + d1 > k) evt = min(evt, t0 + d1);
         };
 
-        // the step at which the running set's earliest or latest
-        // start changes (the last completion among the requests that started at
-        // smin, or at smax)
-        auto window_end = [&]() -> int32_t {
-            int32_t e_lo = INT_MIN, e_hi = INT_MIN;
-#pragma unroll
-            for (int r = 0; r < SPL; ++r)
-                if (busy >> r & 1u) {
-                    if (sa[r] == smin) e_lo = max(e_lo, sc[r]);
-                    if (sa[r] == smax) e_hi = max(e_hi, sc[r]);
-                }
-            return min(__reduce_max_sync(kFull, e_lo), __reduce_max_sync(kFull, e_hi));
-        };
-        // serve steps k .. K - 1 at once, K <= the step at which
-        // the earliest or latest start changes.  Every running request i
-        // (start s_i, completion c_i) runs L_i = min(c_i, K) - k of them, with
-        // max r = t - smin + 1 at step t and r_i = t - s_i + 1:
-        //   W += L_i (k - smin + 1) + L_i (L_i - 1) / 2,  E += L_i (s_i - smin),
-        // and the extent smax - smin is constant.  Requests with c_i < K
-        // complete inside the window and leave here.
+        // Serve steps k .. K - 1 at once, K <= the step at which the earliest or
+        // latest start changes: the extent is constant and max r = t - smin + 1 at
+        // step t, so a request that runs L_i of the steps adds
+        // L_i (k - smin + 1) + L_i (L_i - 1) / 2 to W (max r <= 65535 at each of
+        // them: the sum fits 32 bits).  Those that complete before K leave here.
         auto window = [&](int32_t K) {
-            // twice the W term per slot: L_i (2 m0 - 1 + L_i), m0 = k - smin + 1;
-            // all factors below 2^32
-            const uint32_t m2 = 2u * (uint32_t)(k - smin) + 1u;
-            uint64_t wl2 = 0, el = 0, cl = 0;
-            uint32_t sl = 0;
-            int32_t tl = 0, cmx = 0, nf = 0, of = 0;
-            uint32_t fm = 0u;
-#pragma unroll
-            for (int r = 0; r < SPL; ++r)
-                if (busy >> r & 1u) {
-                    const int32_t c = sc[r];
-                    const uint32_t Li = (uint32_t)(min(c, K) - k);
-                    wl2 += (uint64_t)Li * (m2 + Li);
-                    el += (uint64_t)Li * (uint32_t)(sa[r] - smin);
-                    tl += (int32_t)Li;
-                    if (c < K) {                                  // completes inside the window
-                        const int w = (r << 5) + lane;
-                        fm |= 1u << r;
-                        cl += (uint32_t)c;
-                        sl += (uint32_t)sa[r];
-                        cmx = max(cmx, c);
-                        nf++;
-                        of += S.sres[w];
-                        if (co_out) co_out[S.sjob[w]] = c;
-                        sc[r] = INT_MAX;
-                    }
-                }
-            busy &= ~fm;
-            recompute_lane();
-            W += (int64_t)(warp_sum_u64(wl2) >> 1);             // every slot's term is even
-            E += (int64_t)warp_sum_u64(el);
-            tok += (int32_t)__reduce_add_sync(kFull, (unsigned)tl);
-            nf = (int32_t)__reduce_add_sync(kFull, (unsigned)nf);
-            of = (int32_t)__reduce_add_sync(kFull, (unsigned)of);
-            sumc += (int64_t)warp_sum_u64(cl);
-            sum_st -= __reduce_add_sync(kFull, sl);
-            const int32_t cm = (int32_t)__reduce_max_sync(kFull, (unsigned)cmx);
-            if (nf > 0) Tmake = max(Tmake, cm);
-            done += nf;
-            run_cnt -= nf;
-            kv_sum -= of;
-            kv_over = kv_sum > kv_lim;
-            cmin = __reduce_min_sync(kFull, lane_cmin);
-            const int32_t ext = smax - smin;                  // unchanged inside the window
-            const int32_t L = K - k;
-            sumext += (int64_t)L * ext;
-            maxext = max(maxext, ext);
-            viol += ext > alpha32 ? L : 0;
-            Tb += L;
+            if (kIsjl && plan_left > 0) copy_wait();
+            const uint32_t m0 = (uint32_t)(k - smin) + 1u;
+            const uint32_t thr = (uint32_t)(K - kbase) << RB;
+            uint64_t wl = 0;
+            int32_t freed = 0, nf = 0, cmx = 0;
+            while (key0 < thr) {
+                const int32_t c = kbase + (int32_t)(key0 >> RB);
+                const uint32_t Li = (uint32_t)(c - k);
+                wl += Li * m0 + ((Li * (Li - 1u)) >> 1);
+                cmx = c;                                       // ascending
+                nf++;
+                pop_front(true, freed);
+            }
+            __syncwarp();
+            W += (int64_t)warp_sum_u64(wl);
+            if (trunc) Tmake = max(Tmake, (int32_t)__reduce_max_sync(kFull, (unsigned)cmx));
+            run_cnt -= (int32_t)__reduce_add_sync(kFull, (unsigned)nf);
+            kv_sum -= (int32_t)__reduce_add_sync(kFull, (unsigned)freed);
         };
 
-        // release every request with A_i <= k (a prefix: arrivals are non-decreasing)
         for (;;) {
-            if (k >= step_guard) { status = ISJL_ERR_STEP_LIMIT; break; }   // k > max_steps
-            if (k >= next_arr) release();
-            if (k == cmin) retire(k);
-            if (done == n) break;
-            admit();
-            if (broken) { status = ISJL_ERR_INTERNAL; break; }
-            // next event: arrival, completion or the end of o_1's delay
-            int32_t nxt = min(blocked && run_cnt > 0 ? INT_MAX : next_arr, cmin);
-            if (policy == ISJL_POLICY_ISJL && !L1_started && t0 + d1 > k) nxt = min(nxt, t0 + d1);
-            if (nxt == INT_MAX) { status = ISJL_ERR_STEP_LIMIT; break; }   // cannot progress
-            nxt = min(nxt, step_guard);                          // serve no step past max_steps
+            // ---- steps k .. nxt - 1
+            const uint32_t m = __reduce_min_sync(kFull, key0);
+            const int32_t c = kbase + (int32_t)(m >> RB);        // earliest completion (none: beyond evt)
+            int32_t nxt = min(c, evt);
+            if (min(e_lo, e_hi) <= k) {
+                if (run_cnt > 0) {
+                    rescan();
+                } else {                                         // nothing runs: the steps up to evt are idle
+                    if (P == ISJL_POLICY_FCFS ? fcfs == n : rel == n && pend == 0 && plan_left == 0) break;
+                    if (evt >= (1 << 30) - 1) { status = ISJL_ERR_INTERNAL; break; }   // cannot progress
+                    smin = smax;
+                    nxt = evt;
+                    Tb -= evt - k;
+                }
+            }
+            const int32_t ext = smax - smin;                     // max r - min r
+            const uint32_t m0 = (uint32_t)(k - smin + 1);        // max r at step k
+            if (nxt != k) {
+                peakkv = max(peakkv, kv_sum);
+                peakb = max(peakb, run_cnt);
+            }
             // LJF with a batch running, or ISJL with its gate shut (A_max only
             // grows while the earliest start stays): no request can start
             // before the running set's earliest or latest start changes, so
-            // completions in between end no epoch of their own
-            if (run_cnt > 0 && !kv_over && nxt == cmin &&
-                (policy == ISJL_POLICY_LJF || (policy == ISJL_POLICY_ISJL && k - smin > alpha32))) {
-                const int32_t K = min(window_end(), step_guard);
-                if (K > nxt) {
-                    window(K);
-                    k = K;
-                    continue;
-                }
+            // completions in between end no interval of their own
+            if ((P == ISJL_POLICY_LJF || (kIsjl && k - smin > alpha32)) && run_cnt > 0) {
+                nxt = min(min(e_lo, e_hi), evt_base);
+                window(nxt);
             }
-            if (run_cnt > 0) {
-                // L steps, max r = m0 + t at step k + t, sum r = s m0 - sum (s_i - smin) + s t:
-                //   W += s (L m0 + L (L - 1) / 2),  E += L sum (s_i - smin)
-                // The epoch ends by the completion of the request that started at
-                // smin, so max r <= its o <= 65535 throughout: the sum of max r over
-                // the L <= 65535 steps fits 32 bits, and sum (s_i - smin) <
-                // B * 65536 is exact from the modular sum of starts.
-                const uint32_t L = (uint32_t)(nxt - k), s = (uint32_t)run_cnt;
-                const uint32_t m0 = (uint32_t)(k - smin + 1);     // max r at step k
-                const int32_t ext = smax - smin;                  // max r - min r
-                mad_wide(W, s, L * m0 + ((L * (L - 1u)) >> 1));
-                mad_wide(E, L, sum_st - s * (uint32_t)smin);
-                mad_wide(sumext, L, (uint32_t)ext);
-                maxext = max(maxext, ext);
-                viol += ext > alpha32 ? (int32_t)L : 0;
-                kvviol += kv_over ? (int32_t)L : 0;
-                Tb += (int32_t)L;
-                tok += (int32_t)(s * L);
-            }
+            // L steps, max r = m0 + t at step k + t: W += s (L m0 + L (L - 1) / 2).
+            // The interval ends by the completion of the request that started at
+            // smin, so max r <= its o <= 65535 throughout: the sum of max r over
+            // the L <= 65535 steps fits 32 bits
+            if (nxt < k) { status = ISJL_ERR_INTERNAL; break; }
+            const uint32_t L = (uint32_t)(nxt - k);
+            mad_wide(W, (uint32_t)run_cnt, L * m0 + ((L * (L - 1u)) >> 1));
+            mad_wide(sumext, L, (uint32_t)ext);
+            if (L != 0u) maxext = max(maxext, ext);
+            if (ext > alpha32) viol += (int32_t)L;
+            Tb += (int32_t)L;
             k = nxt;
+            if (k >= min(evt, next_arr)) {
+                if (k >= step_guard) { status = ISJL_ERR_STEP_LIMIT; break; }   // k > max_steps
+                if (RB > 2 && k >= evt_base) {       // keep the keys' relative steps within 32 - RB bits
+                    const uint32_t d = (uint32_t)(k - kbase) << RB;
+#pragma unroll
+                    for (int r = 0; r < SPL; ++r)
+                        if (col[r] != kEmpty) col[r] -= d;
+                    if (key0 != kEmpty) key0 -= d;
+                    kbase = k;
+                    evt_base = (int32_t)min((int64_t)step_guard, (int64_t)k + (1 << 27));
+                }
+                if (k >= next_arr) release();
+            }
+            // ---- requests completing at step k leave.  FCFS, LJF and SJF take one
+            // per lane and pass: a further one at step k leaves in the next pass,
+            // which serves no step, and whatever fits now also fits then
+            const uint32_t thr = ((uint32_t)(k - kbase) << RB) | RM;
+            if (kIsjl && plan_left > 0) copy_wait();
+            int32_t freed = 0;
+            bool f = key0 <= thr;
+            unsigned b = __ballot_sync(kFull, f);
+            if (b) Tmake = k;
+            do {
+                pop_front(f, freed);
+                run_cnt -= __popc(b);
+                if (!kIsjl) break;
+                f = key0 <= thr;
+                b = __ballot_sync(kFull, f);
+            } while (b);
+            kv_sum -= (int32_t)__reduce_add_sync(kFull, (unsigned)freed);
+            // ---- starts
+            admit();
+            if (broken) { status = ISJL_ERR_INTERNAL; break; }
+        }
+        if (kIsjl) copy_wait();
+        if (peakkv > kv_lim) status = ISJL_ERR_INTERNAL;   // every start checks its reservation
+        if (status == ISJL_OK) {
+            tok = (int32_t)is.O;
+            E = W - is.Q;
+            sumc = sums + is.O;                        // sum of starts and true lengths
+        } else {
+            // a request still running has served a = k - s of its o = c - s tokens
+            int64_t rest = 0, run_c = 0;
+            int32_t tok_rest = 0;
+            uint32_t key[SPL];
+            load_column(key);
+#pragma unroll
+            for (int r = 0; r < SPL; ++r)
+                if (key[r] != kEmpty) {
+                    const int32_t c = kbase + (int32_t)(key[r] >> RB);
+                    const int32_t s0 = S.slot[(r << 5) + lane].x;
+                    const uint32_t o = (uint32_t)(c - s0), a = (uint32_t)(k - s0);
+                    rest += (int64_t)((o * (o + 1u)) >> 1) - (int64_t)((a * (a + 1u)) >> 1);
+                    tok_rest += (int32_t)(o - a);
+                    run_c += c;
+                }
+            E = W - warp_sum64((int64_t)R_l - rest);
+            tok = (int32_t)__reduce_add_sync(kFull, (unsigned)(tok_l - tok_rest));
+            sumc = sums + (int64_t)__reduce_add_sync(kFull, (unsigned)tok_l) - warp_sum64(run_c);
+            if (co_out) {
+                __syncwarp();
+                for (int i = lane; i < n; i += 32)
+                    if (status != ISJL_ERR_STEP_LIMIT || co_out[i] >= k) co_out[i] = -1;
+                if (st_out && status != ISJL_ERR_STEP_LIMIT)
+                    for (int i = lane; i < n; i += 32) st_out[i] = -1;
+            }
         }
     }
 
@@ -1028,7 +1122,7 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
         R.sum_extent = sumext;
         R.max_extent = maxext;
         R.violations = viol;
-        R.kv_violations = kvviol;
+        R.kv_violations = 0;   // every start keeps the reservation within the cap
         R.peak_kv = peakkv;
         R.peak_batch = peakb;
         R.status = status;
@@ -1070,24 +1164,22 @@ template <int SPL>
 __global__ void __launch_bounds__(kSimWarpsPerBlock * 32, sim_min_blocks<SPL>())
 sim_kernel(SimArgs A, int64_t n_tasks) {
     extern __shared__ __align__(16) int32_t smem[];
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    const int per = smem_words_per_warp(A.B, A.words0, A.words1);
+    const int lane = threadIdx.x & 31, wib = (int)__reduce_max_sync(kFull, threadIdx.x >> 5);
+    const int per = smem_words_per_warp(SPL, A.B, A.words0, A.words1);
     int32_t *b = smem + (size_t)wib * per;
     WarpSmem S;
-    S.sjob = b;
-    S.shead = b + A.B;
-    S.stail = b + 2 * A.B;
+    S.key = reinterpret_cast<uint32_t *>(b);
+    b += 32 * SPL;
+    S.slot = reinterpret_cast<int2 *>(b);
+    S.slink = reinterpret_cast<uint32_t *>(b + 2 * A.B);
     S.slong = b + 3 * A.B;
-    S.srem = b + 4 * A.B;
-    S.spsum = b + 5 * A.B;
-    S.sres = b + 6 * A.B;
-    S.pend0 = reinterpret_cast<uint32_t *>(b + 7 * A.B);
+    S.pend0 = reinterpret_cast<uint32_t *>(b + 4 * A.B);
     S.pend1 = S.pend0 + A.words0;
     const int64_t gwarp = (int64_t)blockIdx.x * kSimWarpsPerBlock + wib;
     for (;;) {
         int t = 0;
         if (lane == 0) t = atomicAdd(A.task_counter, 1);
-        t = __shfl_sync(kFull, t, 0);
+        t = (int)__reduce_max_sync(kFull, (unsigned)t);
         if ((int64_t)t >= n_tasks) break;
         // run-major: at any time the warps of an SM mostly run one policy's code
         const int64_t inst = t % A.n_inst;
@@ -1124,7 +1216,7 @@ int slots_per_lane(int B) {
 
 size_t sim_smem_per_warp(int B, int n) {
     const int words0 = (n + 31) / 32, words1 = (words0 + 31) / 32;
-    return (size_t)smem_words_per_warp(B, words0, words1) * 4;
+    return (size_t)smem_words_per_warp(slots_per_lane(B), B, words0, words1) * 4;
 }
 
 static cudaError_t occupancy(int B, int n, int device, int *blocks_per_sm, int *sms, size_t *smem) {
