@@ -1,0 +1,43 @@
+"""Batches of completions on the GPU against the oracle: runs whose queue head
+waits for KV or a slot, at the sizes and lengths where a batch has to stop or to
+fall back (more than 32 completions at one step, requests shorter than the
+batch, one slot, every row count, slack, a step guard inside a batch)."""
+import numpy as np
+import pytest
+
+from conftest import cuda_available
+from test_parity_gpu import INF, O, S, run_both  # noqa: F401  (fixtures)
+
+pytestmark = [pytest.mark.gpu, pytest.mark.skipif(not cuda_available(), reason="needs a CUDA GPU")]
+
+POLICIES = ["fcfs"]
+
+
+def lengths(rng, kind, shape):
+    if kind == "ties":                      # whole batches complete at one step
+        return rng.choice(np.array([40, 40, 40, 41], np.int32), shape).astype(np.int32)
+    if kind == "short":                     # many requests end before the batch they start in
+        return np.where(rng.random(shape) < 0.5, rng.integers(1, 4, shape), rng.integers(100, 900, shape)).astype(
+            np.int32)
+    if kind == "long":                      # lengths up to the limit
+        return np.minimum(rng.pareto(1.1, shape) * 300 + 1, 65_535).astype(np.int32)
+    return rng.integers(1, 2000, shape).astype(np.int32)
+
+
+@pytest.mark.parametrize("policy", POLICIES)
+@pytest.mark.parametrize("kind", ["ties", "short", "long", "mixed"])
+@pytest.mark.parametrize("B", [1, 5, 32, 33, 64, 128, 200, 512])
+def test_batches_of_completions(S, O, policy, kind, B):  # noqa: F811
+    rng = np.random.default_rng(100 + B)
+    n = 700
+    o = lengths(rng, kind, (3, n))
+    p = np.zeros_like(o)
+    a = np.zeros_like(o)
+    a[1] = np.sort(rng.integers(0, 300, n))
+    a[2] = np.sort(rng.integers(0, 20_000, n))          # queue empty now and then
+    big = int(o.max())
+    for kv, slack, ms in [(INF, None, 0), (max(big, int(o.mean() * B * 0.6)), None, 0),
+                          (big + 40, rng.integers(0, 40, o.shape).astype(np.int32), 0), (big * 3, None, 997)]:
+        if slack is not None:
+            o = np.minimum(o, 65_535 - 40)
+        run_both(S, O, a, p, o, B, [policy], [50], kv, False, slack=slack, max_steps=ms)
