@@ -34,6 +34,7 @@
 // request is the lowest set bit -- with a summary word per 32 words, in shared
 // memory.  ISJL plans are per-worker FIFO lists linked through a global
 // scratch array.
+#include <algorithm>
 #include <climits>
 #include <cstdint>
 
@@ -43,6 +44,9 @@ namespace isjl {
 namespace {
 
 constexpr int32_t kNone = -1;
+// ISJL whose budget no request's length exceeds: it never plans (o_2 <= alpha) and
+// its gate never shuts, so it starts the longest pending request that fits
+constexpr int kPolicyLpt = ISJL_POLICY_ISJL_BETA + 1;
 constexpr uint32_t kEmpty = 0xFFFFFFFFu;   // key of a slot that holds no running request
 
 // bits of a running request's key that hold its register row
@@ -112,6 +116,7 @@ __device__ __forceinline__ int bs_next(const WarpSmem &S, int words0, int words1
         const int ww = (w1 << 5) + __ffs(u) - 1;
         return (ww << 5) + __ffs(S.pend0[ww]) - 1;
     }
+#pragma unroll 1
     for (int b1 = w1 + 1; b1 < words1; b1 += 32) {
         const int idx = b1 + lane;
         const uint32_t x = idx < words1 ? S.pend1[idx] : 0u;
@@ -138,6 +143,7 @@ __device__ __forceinline__ void bs_clear(const WarpSmem &S, int p, int lane) {
 
 // highest pending sorted position, -1 if none (uniform call)
 __device__ __forceinline__ int bs_last(const WarpSmem &S, int words1, int lane) {
+#pragma unroll 1
     for (int b1 = (words1 - 1) & ~31; b1 >= 0; b1 -= 32) {
         const int idx = b1 + lane;
         const uint32_t x = idx < words1 ? S.pend1[idx] : 0u;
@@ -183,6 +189,7 @@ __device__ __forceinline__ int nth_set_bit(uint32_t x, int k) {
 __device__ __forceinline__ int bs_count_below(const WarpSmem &S, int words0, int P, int lane) {
     const int full = P >> 5;
     int cnt = 0;
+#pragma unroll 1
     for (int w = lane; w < full && w < words0; w += 32) cnt += __popc(S.pend0[w]);
     if (lane == 0 && (P & 31) && full < words0) cnt += __popc(S.pend0[full] & ((1u << (P & 31)) - 1u));
     return (int)__reduce_add_sync(kFull, (unsigned)cnt);
@@ -195,6 +202,7 @@ __device__ __forceinline__ int bs_count_below(const WarpSmem &S, int words0, int
 // four, instead of a binary search's 10 and 17.
 __device__ __forceinline__ int first_pos_le(const int32_t *os, int n, int64_t x, int lane) {
     int lo = 0, hi = n;                         // the answer lies in [lo, hi]
+#pragma unroll 1
     while (hi - lo > 32) {
         const int step = (hi - lo + 31) >> 5;
         const int idx = lo + lane * step;
@@ -211,9 +219,23 @@ __device__ __forceinline__ int first_pos_le(const int32_t *os, int n, int64_t x,
     return b ? lo + __ffs(b) - 1 : lo + 32;
 }
 
+// v as a value the optimiser cannot see through.  A condition that holds for a
+// whole task (which outputs there are, whether lengths are predictions) would
+// otherwise have the event loop compiled once for each of its outcomes, and the
+// copies crowd each other out of the instruction cache: a task runs most of its
+// code only a few times, so ISJL's runs are bound by instruction fetch.  (With
+// this, with short loops rolled and with one pass over the rows per completion
+// window, ISJL's body went from 104 to 76 KB; 100,000 x 500 requests under 5 runs
+// from 29.8 to 23.6 ms, the profit experiment from 3.56 to 2.57 ms.)
+__device__ __forceinline__ int opaque(int v) {
+    asm volatile("" : "+r"(v));
+    return v;
+}
+
 // One (instance, run) task under policy P, a compile-time constant (FCFS, LJF,
-// SJF or ISJL; Algorithm "ISJL" runs the ISJL body with beta in the packing
-// thresholds), so each policy's code holds only its own admission rule.
+// SJF, ISJL or ISJL without a binding budget; Algorithm "ISJL" runs the ISJL body
+// with beta in the packing thresholds), so each policy's code holds only its own
+// admission rule.
 //
 // Running requests.  Worker w = r * 32 + lane owns slot row r of its lane.  A
 // slot's key is the completion step (relative to kbase) above lane and row; a
@@ -248,8 +270,9 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
     constexpr uint32_t RM = (1u << RB) - 1u;
     constexpr int SH = RB + 5;                      // a key's completion step lies above lane and row
     constexpr int32_t kSpan = 1 << (30 - SH);       // kbase follows k when it is this far behind
-    constexpr bool kBatch = P == ISJL_POLICY_FCFS;
     constexpr bool kIsjl = P == ISJL_POLICY_ISJL;
+    constexpr bool kLpt = P == kPolicyLpt;
+    constexpr bool kBatch = P == ISJL_POLICY_FCFS || kLpt;
     const int n_slots = A.n, B = A.B;
     const int64_t base = inst * (int64_t)n_slots;
     const InstStats is = A.inst[inst];
@@ -275,9 +298,14 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
     // every schedule ends by sum o + max arrival; completion steps need < 2^30
     if (status == ISJL_OK && is.O + (int64_t)is.maxA + 1 >= (int64_t)(1 << 30)) status = ISJL_ERR_INVALID_ARG;
     const bool trunc = A.max_steps > 0;             // the run may be stopped early
+    // conditions of the whole task, tested through opaque()
+    const int kHasStart = 1, kHasCompl = 2, kTrunc = 4, kSlack = 8, kPacked = 16;
+    const int flags = (st_out ? kHasStart : 0) | (co_out ? kHasCompl : 0) | (trunc ? kTrunc : 0) |
+                      (otru ? kSlack : 0) | (n_slots <= 65536 ? kPacked : 0);
     // requests that never start / finish report -1: all of them on an error
     // status (and to begin with in a run that may be stopped), else the unused
     // slots of a ragged instance (a full run writes every other entry)
+#pragma unroll 1
     for (int i = (status != ISJL_OK || trunc ? 0 : n) + lane; i < n_slots; i += 32) {
         if (st_out) st_out[i] = -1;
         if (co_out) co_out[i] = -1;
@@ -289,7 +317,9 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
 
     if (status == ISJL_OK && n > 0) {
         if (P != ISJL_POLICY_FCFS) {
+#pragma unroll 1
             for (int w = lane; w < words0; w += 32) S.pend0[w] = 0u;
+#pragma unroll 1
             for (int w = lane; w < words1; w += 32) S.pend1[w] = 0u;
         }
         __syncwarp();
@@ -355,7 +385,7 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
             hw = 0u;
             if (i < n) {
                 const uint32_t u = (uint32_t)oarr[i];
-                hw = (u << 16) | (otru ? (uint32_t)otru[i] : u);
+                hw = (u << 16) | ((opaque(flags) & kSlack) ? (uint32_t)otru[i] : u);
             }
         };
         if (P == ISJL_POLICY_FCFS) {
@@ -370,6 +400,13 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
         // start range of the running set and the last completions of those started
         // at its ends; found again (rescan) once e_lo or e_hi is reached
         int32_t smin = 0, smax = 0, e_lo = INT_MIN, e_hi = INT_MIN;
+        // Batches of completions (below): the smallest keys in ascending order, lane i
+        // the i-th of nn (kEmpty beyond); every other key's step is at least near_end
+        uint32_t nk = kEmpty;
+        int nn = 0, span = 64, skip = 0;
+        int32_t near_end = 0;
+        bool stale = false;                            // key0 is to be reloaded
+
         int32_t plan_left = 0, t0 = 0, d1 = 0, nlong = 0;
         bool L1_started = true;
         bool broken = false;   // an internal invariant failed: stop without touching memory
@@ -381,12 +418,12 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
 
         // plan links: request and planning length of the entry after a request,
         // in one word when request indices fit 16 bits, else the index plus one
-        const bool packed = n_slots <= 65536;
+        auto packed = [&]() -> bool { return opaque(flags) & kPacked; };
         auto link_of = [&](int e, int oe) -> uint32_t {
-            return packed ? ((uint32_t)oe << 16) | (uint32_t)e : (uint32_t)e + 1u;
+            return packed() ? ((uint32_t)oe << 16) | (uint32_t)e : (uint32_t)e + 1u;
         };
-        auto link_job = [&](uint32_t lk) -> int { return packed ? (int)(lk & 0xFFFFu) : (int)(lk - 1u); };
-        auto link_len = [&](uint32_t lk) -> int { return packed ? (int)(lk >> 16) : oarr[lk - 1u]; };
+        auto link_job = [&](uint32_t lk) -> int { return packed() ? (int)(lk & 0xFFFFu) : (int)(lk - 1u); };
+        auto link_len = [&](uint32_t lk) -> int { return packed() ? (int)(lk >> 16) : oarr[lk - 1u]; };
 
         // this lane starts request e (planning length oe, true length oc) in slot
         // row `row` at step k
@@ -394,9 +431,10 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
             const int c = k + oc;
             idle &= ~(1u << row);
             S.slot[(row << 5) + lane] = make_int2(k, oe);
-            if (st_out) st_out[e] = k;
-            if (co_out) co_out[e] = c;
-            if (trunc) {
+            const int f = opaque(flags);
+            if (f & kHasStart) st_out[e] = k;
+            if (f & kHasCompl) co_out[e] = c;
+            if (f & kTrunc) {
                 R_l += ((uint32_t)oc * (uint32_t)(oc + 1)) >> 1;      // oc (oc + 1) < 2^32
                 tok_l += oc;
             }
@@ -407,9 +445,16 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
         // warp-wide totals of cnt starts at step k that reserve kv_add and whose
         // last completion is c_hi
         auto commit = [&](int cnt, int32_t kv_add, int32_t c_hi) {
+            nn = 0;
             run_cnt += cnt;
             kv_sum += kv_add;
             mad_wide(sums, (uint32_t)cnt, (uint32_t)k);
+            if (run_cnt == cnt) {                          // nothing was running
+                smin = k;
+                e_lo = c_hi;
+            } else if (smin == k) {
+                e_lo = max(e_lo, c_hi);
+            }
             e_hi = smax == k ? max(e_hi, c_hi) : c_hi;
             smax = k;
         };
@@ -438,8 +483,9 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
             const bool fit = lane < m && lane < nfree && kv_sum + pre <= kv_lim;
             const int c = __popc(__ballot_sync(kFull, fit));
             if (c == 0) return 0;
-            const int oc_l = (otru && lane < c) ? otru[ce] : co;  // it finishes after its true length
+            const int oc_l = ((opaque(flags) & kSlack) && lane < c) ? otru[ce] : co;  // it finishes after its true length
             const int32_t c_hi = k + (int32_t)__reduce_max_sync(kFull, lane < c ? (unsigned)oc_l : 0u);
+#pragma unroll 1
             for (int placed = 0; placed < c;) {                   // one per lane with a free slot and round
                 const bool f = fm != 0u;
                 const unsigned b = __ballot_sync(kFull, f);
@@ -458,28 +504,28 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
             return c;
         };
 
-        // the earliest request of this lane's column leaves if f; freed += its KV
-        auto pop_front = [&](bool f, int32_t &freed) {
-            const uint32_t row = key0 & RM;
+        // the request on this lane's slot row `row` leaves; freed += its KV
+        auto vacate = [&](uint32_t row, int32_t &freed) {
             const int w = (int)(row << 5) + lane;
-            if (f) {
-                freed += S.slot[w].y;
-                if (kIsjl && plan_left > 0) {
-                    const uint32_t lk = S.slink[w];
-                    if (lk) {                                 // the worker's next plan entry waits now
-                        resv |= 1u << row;
-                        if (!L1_started && w < nlong && link_job(lk) == S.slong[w]) lhead |= 1u << row;
-                    }
+            freed += S.slot[w].y;
+            if (kIsjl && plan_left > 0) {
+                const uint32_t lk = S.slink[w];
+                if (lk) {                                     // the worker's next plan entry waits now
+                    resv |= 1u << row;
+                    if (!L1_started && w < nlong && link_job(lk) == S.slong[w]) lhead |= 1u << row;
                 }
             }
-            if (f) {
-                idle |= 1u << row;
-                if (SPL > 1) {
-                    col[row] = kEmpty;
-                    column_min();
-                } else {
-                    key0 = kEmpty;
-                }
+            idle |= 1u << row;
+        };
+        // this lane's earliest request leaves
+        auto pop_front = [&](int32_t &freed) {
+            const uint32_t row = key0 & RM;
+            vacate(row, freed);
+            if (SPL > 1) {
+                col[row] = kEmpty;
+                column_min();
+            } else {
+                key0 = kEmpty;
             }
         };
         // start range of the running set, and the last completions at its ends
@@ -514,11 +560,26 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
             if (p >= 0 && p < n) {
                 ho = osrt[p];
                 he = perm[p];
-                ht = otru ? otru[he] : ho;
+                ht = (opaque(flags) & kSlack) ? otru[he] : ho;
             }
         };
         // requests with A_i <= k join the queue (a prefix: arrivals are non-decreasing)
         auto release = [&]() {
+            if (P != ISJL_POLICY_FCFS && rel == 0 && is.maxA <= k) {   // all of them at once
+#pragma unroll 1
+                for (int b = 0; b < words0; b += 32) {
+                    const int i = b + lane;
+                    if (i < words0) S.pend0[i] = i + 1 < words0 || (n & 31) == 0 ? ~0u : (1u << (n & 31)) - 1u;
+                    if (i < words1) S.pend1[i] = i + 1 < words1 || (words0 & 31) == 0 ? ~0u : (1u << (words0 & 31)) - 1u;
+                }
+                rel = n;
+                pend = n;
+                next_arr = INT_MAX;
+                __syncwarp();
+                set_head(P == ISJL_POLICY_SJF ? n - 1 : 0);
+                return;
+            }
+#pragma unroll 1
             for (;;) {
                 // released: window lanes at or after rel whose arrival is <= k (a prefix)
                 const bool ok = win_base + lane >= rel && win_a <= k;
@@ -564,6 +625,7 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
         // (uniform call)
         auto first_pending_from = [&](int p0, int m) -> int {
             int mine = -1;
+#pragma unroll 1
             for (int wb = (p0 >> 10) << 5, got = 0; got < m && wb < words0; wb += 32) {
                 if (S.pend1[wb >> 5] == 0u) continue;           // no pending in these 32 words
                 const int wi = wb + lane;
@@ -604,10 +666,12 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
         // idle slots (ISJL: not reserved for a plan entry) until one does not fit
         // or the slots run out
         auto start_longest = [&]() {
-            // one at a time for the first two starts (usually all there are),
-            // then 32 at a time; every round first checks that the head fits
+            // one at a time for the first two starts (usually all there are unless
+            // nothing runs), then 32 at a time; every round first checks that the
+            // head fits
             unsigned lanes = __ballot_sync(kFull, (idle & ~resv) != 0u);
-            for (int nseq = 0; pend > 0 && kv_sum + ho <= kv_lim && lanes != 0u; ++nseq) {
+#pragma unroll 1
+            for (int nseq = run_cnt == 0 ? 2 : 0; pend > 0 && kv_sum + ho <= kv_lim && lanes != 0u; ++nseq) {
                 if (hp >= n) { broken = true; return; }
                 if (nseq < 2) {
                     start_any(he, ho, ht, idle & ~resv, lanes);
@@ -638,7 +702,7 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
             int c = 0;
             int32_t kv_add = 0;
             uint32_t oc_hi = 0u;
-#pragma unroll
+#pragma unroll 1
             for (int r = 0; r < SPL; ++r) {
                 const bool el = !stopped && (cand >> r & 1u);
                 if (__ballot_sync(kFull, el) != 0u) {
@@ -649,24 +713,27 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
                         e = link_job(lk);
                         oe = link_len(lk);
                     }
-                    int pre = oe;                               // prefix over this row, in lane order
-#pragma unroll
-                    for (int d = 1; d < 32; d <<= 1) {
-                        const int t = __shfl_up_sync(kFull, pre, d);
-                        if (lane >= d) pre += t;
+                    bool fits = el;
+                    const int row_kv = (int)__reduce_add_sync(kFull, (unsigned)oe);
+                    if (kv_sum + kv_add + row_kv > kv_lim) {
+                        int pre = oe;                           // prefix over this row, in lane order
+#pragma unroll 1
+                        for (int d = 1; d < 32; d <<= 1) {
+                            const int t = __shfl_up_sync(kFull, pre, d);
+                            if (lane >= d) pre += t;
+                        }
+                        fits = el && kv_sum + kv_add + pre <= kv_lim;
+                        stopped = true;                         // the first one that does not fit
                     }
-                    const bool fits = el && kv_sum + kv_add + pre <= kv_lim;
-                    const unsigned fb = __ballot_sync(kFull, fits);
-                    if (fb != __ballot_sync(kFull, el)) stopped = true;   // the first one that does not fit
                     if (fits) {
                         copy_async(S.slink + w, pnext + e);
-                        const int oc = otru ? otru[e] : oe;     // it finishes after its true length
+                        const int oc = (opaque(flags) & kSlack) ? otru[e] : oe;     // it finishes after its true length
                         occupy(e, oe, oc, r);
                         resv &= ~(1u << r);
                         lhead &= ~(1u << r);
                         oc_hi = max(oc_hi, (uint32_t)oc);
                     }
-                    c += __popc(fb);
+                    c += __popc(__ballot_sync(kFull, fits));
                     kv_add += (int32_t)__reduce_add_sync(kFull, fits ? (unsigned)oe : 0u);
                 }
             }
@@ -677,9 +744,9 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
         };
 
         // ISJL Phase ONE at a stage start (Algorithm 2 with beta = alpha).  Nothing
-        // runs, so the slots' array is free: it holds each worker's last plan entry and
-        // first its packing budget, then its pack sum; room[] holds the packing
-        // budgets left (0: takes no pack)
+        // runs, so the slots' arrays are free: slot[] holds each worker's last plan entry
+        // and first its packing budget, then its pack sum, the key columns hold the
+        // packing budgets left (0: takes no pack)
         auto phase_one = [&]() {
             const int64_t alpha = A.runs.delta[run], beta = A.runs.beta[run];
             t0 = k; d1 = 0; L1_started = true; nlong = 0;
@@ -696,6 +763,7 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
             const int nl = min(B, cnt_long);
             copy_wait();                                        // links of the last stage still in flight
             __syncwarp();
+#pragma unroll 1
             for (int w = lane; w < B; w += 32) {
                 S.slot[w] = make_int2(kNone, w >= nl ? (int32_t)alpha : 0);   // workers M+1..B: alpha
                 S.slink[w] = 0u;
@@ -706,6 +774,7 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
             // worker j's budget cap_j.  Up to 32 at a time: a prefix sum of the
             // bitset words' popcounts gives each lane the word and bit of its rank
             int olast_l = 0;
+#pragma unroll 1
             for (int wb = 0, taken = 0; taken < nl; wb += 32) {
                 if (wb >= words0) { broken = true; return; }
                 const int wi = wb + lane;
@@ -719,6 +788,7 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
                 }
                 const int excl = incl - c;
                 const int m = min(nl - taken, __shfl_sync(kFull, incl, 31));   // ranks from this chunk
+#pragma unroll 1
                 for (int r0 = 0; r0 < m; r0 += 32) {
                     const int jj = r0 + lane;                       // rank within the chunk
                     int lo = 0;                                     // lanes whose words end before it
@@ -754,32 +824,33 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
             const int64_t o_last = __reduce_max_sync(kFull, olast_l);
             pend -= nl;
             const int64_t theta = min(2 * alpha, o1 - o_last + beta);
-            uint32_t room[SPL];
-#pragma unroll
+            auto give = [&](int r, uint32_t v) { if (SPL > 1) col[r] = v; else key0 = v; };
+            auto has_room = [&](int r) -> uint32_t { return SPL > 1 ? col[r] : key0; };
+            // this lane's rows whose worker takes no long request (M+1..B)
+            uint32_t rows_short = 0u;
+#pragma unroll 1
             for (int r = 0; r < SPL; ++r) {
                 const int w = (r << 5) + lane;
-                room[r] = w < B ? (uint32_t)S.slot[w].y : 0u;
+                give(r, w < B ? (uint32_t)S.slot[w].y : 0u);
                 if (w < B) S.slot[w].y = 0;
+                rows_short |= (uint32_t)(w >= nl) << r;
             }
             __syncwarp();
-            // maxrem bounds the largest budget from above; it is recomputed only
+            // x bounds the sizes that may still fit from above; it is recomputed only
             // when a candidate no larger than it fits nowhere (budgets only shrink)
             auto max_budget = [&]() -> int {
                 uint32_t m = 0u;
-#pragma unroll
-                for (int r = 0; r < SPL; ++r) m = max(m, room[r]);
+#pragma unroll 1
+                for (int r = 0; r < SPL; ++r) m = max(m, has_room(r));
                 return (int)__reduce_max_sync(kFull, m);
             };
             int64_t x = min(theta, (int64_t)max_budget());
-            // this lane's rows whose worker takes no long request (M+1..B)
-            uint32_t rows_short = 0u;
-#pragma unroll
-            for (int r = 0; r < SPL; ++r) rows_short |= (uint32_t)((r << 5) + lane >= nl) << r;
             // First fit of the shorter requests, in sorted order, on workers M+1..B
             // first, then M, M-1, ..., 2.  32 candidates at a time: lane l loads the
             // l-th; each is placed by a search over all budgets, and the plan lists
             // are linked once per 32
             int from = x >= 1 ? first_pos_le(osrt, n, x, lane) : n;
+#pragma unroll 1
             while (x >= 1 && from < n) {
                 const int q = first_pending_from(from, 32);
                 const int last = __reduce_max_sync(kFull, q);
@@ -789,11 +860,14 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
                 int wsel = -1 - lane;                           // the worker it goes to (distinct if none)
                 bool shrunk = false;
                 unsigned todo = __ballot_sync(kFull, (int64_t)oe <= x);
+#pragma unroll 1
                 while (todo) {
                     const int i = __ffs(todo) - 1;
                     todo &= todo - 1u;
                     const uint32_t o = (uint32_t)__shfl_sync(kFull, oe, i);
                     uint32_t fit = 0u;                          // rows whose budget takes it
+                    uint32_t room[SPL];
+                    load_column(room);
 #pragma unroll
                     for (int r = 0; r < SPL; ++r) fit |= (uint32_t)(room[r] >= o) << r;
                     // code of this lane's first choice: w for a short worker, 1023 - w for a long one
@@ -809,9 +883,7 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
                         continue;
                     }
                     const int w = code < 512u ? (int)code : 1023 - (int)code;
-                    const uint32_t dec = lane == (w & 31) ? o : 0u;   // the chosen worker's budget shrinks
-#pragma unroll
-                    for (int r = 0; r < SPL; ++r) room[r] -= r == (w >> 5) ? dec : 0u;
+                    if (lane == (w & 31)) give(w >> 5, has_room(w >> 5) - o);   // the chosen worker's budget shrinks
                     if (lane == i) wsel = w;
                 }
                 // append the window's requests to their workers' lists, in lane order
@@ -843,10 +915,11 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
                 if (shrunk && x >= 1) from = max(from, first_pos_le(osrt, n, x, lane));
             }
             // worker j (2..M) runs o_j after its pack
+#pragma unroll 1
             for (int w = 1 + lane; w < nl; w += 32) {
                 const int e = S.slong[w];
                 const int tl = S.slot[w].x;
-                const uint32_t lk = link_of(e, packed ? oarr[e] : 0);
+                const uint32_t lk = link_of(e, packed() ? oarr[e] : 0);
                 if (tl < 0) S.slink[w] = lk; else pnext[tl] = (int32_t)lk;
                 pnext[e] = 0;
             }
@@ -855,17 +928,20 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
             plan_left += nl;
             // o_1 waits d1 = min{max{max_j sum(w_j) - alpha, 0}, alpha}, j = 2..M
             int mx = 0;
+#pragma unroll 1
             for (int w = 1 + lane; w < nl; w += 32) mx = max(mx, S.slot[w].y);
             mx = __reduce_max_sync(kFull, mx);
             d1 = (int32_t)min(max((int64_t)mx - alpha, (int64_t)0), alpha);
             resv = 0u;
             lhead = 0u;
-#pragma unroll
+#pragma unroll 1
             for (int r = 0; r < SPL; ++r) {
                 const int w = (r << 5) + lane;
-                if (w < B && S.slink[w]) {
+                give(r, kEmpty);
+                const uint32_t lk = w < B ? S.slink[w] : 0u;
+                if (lk) {
                     resv |= 1u << r;
-                    if (w >= 1 && w < nl && link_job(S.slink[w]) == S.slong[w]) lhead |= 1u << r;
+                    if (w >= 1 && w < nl && link_job(lk) == S.slong[w]) lhead |= 1u << r;
                 }
             }
             L1_started = false;
@@ -873,13 +949,6 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
             __syncwarp();
             set_head(bs_next(S, words0, words1, 0, lane));   // Phase ONE removed queued requests
         };
-
-        // Batches of completions (below): the smallest keys in ascending order, lane i
-        // the i-th of nn (kEmpty beyond); every other key's step is at least near_end
-        uint32_t nk = kEmpty;
-        int nn = 0, span = 64, skip = 0;
-        int32_t near_end = 0;
-        bool stale = false;                            // key0 is to be reloaded
 
         // After an admission, `blocked` says that no arrival alone can let a
         // request start before the next completion (or o_1's delay expiry):
@@ -895,9 +964,9 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
                 // arrival order; the first request that does not fit ends the step;
                 // one at a time for the first two starts (usually all there are),
                 // then 32 at a time
+#pragma unroll 1
                 for (int nseq = 0; fcfs < rel && kv_sum + (int)(fh >> 16) <= kv_lim && run_cnt < B; ++nseq) {
                     int c = 1;
-                    nn = 0;
                     if (nseq < 2) {
                         start_any(fcfs, (int)(fh >> 16), (int)(fh & 0xFFFFu), idle, __ballot_sync(kFull, idle != 0u));
                     } else {
@@ -915,6 +984,7 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
                 // pending positions from the first of that length upwards, in start
                 // order; one at a time for the first two starts, then up to 32 of
                 // them at a time
+#pragma unroll 1
                 for (int nseq = 0; pend > 0 && kv_sum + ho <= kv_lim && run_cnt < B; ++nseq) {
                     if (hp < 0 || hp >= n) { broken = true; return; }
                     // first position of this length: usually among the 32 up to hp
@@ -925,7 +995,7 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
                         const int p = bs_next(S, words0, words1, g, lane);
                         if (p > hp) { broken = true; return; }
                         const int e = p == hp ? he : perm[p];
-                        const int oc = otru ? otru[e] : ho;
+                        const int oc = (opaque(flags) & kSlack) ? otru[e] : ho;
                         start_any(e, ho, oc, idle, __ballot_sync(kFull, idle != 0u));
                         bs_clear(S, p, lane);
                         pend--;
@@ -945,16 +1015,15 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
                 // static batch of the longest released requests when nothing runs
                 if (run_cnt == 0) start_longest();
                 blocked = run_cnt != 0;
+            } else if (kLpt) {
+                start_longest();
+                blocked = pend > 0;
             } else {
                 if (run_cnt == 0 && plan_left == 0 && pend > 0) phase_one();
                 if (broken) return;
-                // the gate A_max(k) <= alpha; progress stays below o <= 65535, so a
-                // budget of at least 65535 never shuts it
+                // the gate A_max(k) <= alpha
                 bool stop = false;
-                if (alpha32 < 65535 && run_cnt > 0) {
-                    if (e_lo <= k) rescan();
-                    stop = k - smin > alpha32;
-                }
+                if (run_cnt > 0) stop = k - smin > alpha32;
                 if (!stop && plan_left > 0) {
                     // plan starts, workers in order; entries that must wait (o_1's
                     // delay, o_j before o_1) are filtered out up front
@@ -963,6 +1032,7 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
                         cand &= ~lhead;
                         if (k < t0 + d1 && lane == 0) cand &= ~1u;   // worker 0 holds o_1
                     }
+#pragma unroll 1
                     for (int nseq = 0; __ballot_sync(kFull, cand != 0u) != 0u; ++nseq) {
                         if (nseq >= 2) {                            // the rest at once
                             stop = plan_bulk(cand);
@@ -986,7 +1056,7 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
                             L1_started = true;
                             cand |= lhead;
                         }
-                        start(e, oe, otru ? otru[e] : oe, owner, row);
+                        start(e, oe, (opaque(flags) & kSlack) ? otru[e] : oe, owner, row);
                     }
                 }
                 if (!stop) start_longest();   // Phase TWO: longest released first
@@ -1007,23 +1077,35 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
             const uint32_t thr = (uint32_t)(K - kbase) << SH;
             uint64_t wl = 0;
             int32_t freed = 0, nf = 0, cmx = 0;
-            while (key0 < thr) {
-                const int32_t c = kbase + (int32_t)(key0 >> SH);
-                const uint32_t Li = (uint32_t)(c - k);
-                wl += Li * m0 + ((Li * (Li - 1u)) >> 1);
-                cmx = c;                                       // ascending
-                nf++;
-                pop_front(true, freed);
+            uint32_t least = kEmpty;
+#pragma unroll 1
+            for (int r = 0; r < SPL; ++r) {
+                const uint32_t x = SPL > 1 ? col[r] : key0;
+                if (x < thr) {
+                    const int32_t c = kbase + (int32_t)(x >> SH);
+                    const uint32_t Li = (uint32_t)(c - k);
+                    wl += Li * m0 + ((Li * (Li - 1u)) >> 1);
+                    cmx = max(cmx, c);
+                    nf++;
+                    vacate(r, freed);
+                    if (SPL > 1) col[r] = kEmpty;
+                } else {
+                    least = min(least, x);
+                }
             }
+            key0 = least;
             __syncwarp();
             W += (int64_t)warp_sum_u64(wl);
-            if (trunc) Tmake = max(Tmake, (int32_t)__reduce_max_sync(kFull, (unsigned)cmx));
+            if (opaque(flags) & kTrunc) Tmake = max(Tmake, (int32_t)__reduce_max_sync(kFull, (unsigned)cmx));
             run_cnt -= (int32_t)__reduce_add_sync(kFull, (unsigned)nf);
             kv_sum -= (int32_t)__reduce_add_sync(kFull, (unsigned)freed);
+            nn = 0;
         };
 
-        // ---- Batches of completions.  While the queue head waits for KV or a slot,
-        // nothing but completions lets a request start.  The next up to 32
+        // ---- Batches of completions (FCFS, and ISJL without a binding
+        // budget).  While the queue head waits for KV or a slot, nothing but completions
+        // lets a request start (longest first: until the next arrival, which may be
+        // longer than the head).  The next up to 32
         // completions (i, ascending) and the next up to 31 queued requests (j, in
         // start order) are then served in one pass: with F the prefix sums of the KV
         // that the completions free and P those of the KV that the requests need,
@@ -1036,6 +1118,10 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
         // 0.42 us (FCFS over a 20,000-request trace); batched, 45 and 0.13 us.  FCFS
         // alone, before -> after: 10,000 x 1,000 requests 2.74 -> 1.32 ms, 100,000 x
         // 500 9.6 -> 5.0 ms, 1,024 x 100,000 45 -> 12.7 ms.
+        // Longest first, 10,000 x 1,000 requests: 4.6 -> 3.3 ms.  ISJL with a binding
+        // budget has no such pass: its plan and gate leave few completions in a row
+        // (a pass for its plan entries, tried, made its body 15% larger and the sweeps
+        // 13 to 26% slower).
 
         // collect the next completions: those within the next `span` steps, a number
         // of steps kept such that there are 16 to 32 where so many run
@@ -1052,11 +1138,13 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
                 return (int)__reduce_add_sync(kFull, (unsigned)mine);
             };
             int c = count(span), over = 0, at = span;   // over: a span with too many, if known
+#pragma unroll 1
             while (c > 32) {
                 over = span;
                 at = span >>= 1;
                 c = count(span);
             }
+#pragma unroll 1
             while (over == 0 && c < 16 && c < run_cnt && span < 65536) {
                 at = 2 * span;
                 const int c2 = count(at);
@@ -1064,6 +1152,7 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
                 span = at;
                 c = c2;
             }
+#pragma unroll 1
             while (over != 0 && c < 8 && over - span > 1) {
                 at = (span + over) >> 1;
                 const int c2 = count(at);
@@ -1114,7 +1203,10 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
                 if (lane >= nn) nk = kEmpty;
             }
         };
-        auto waits = [&]() -> bool { return fcfs < rel && run_cnt > 0; };
+        auto waits = [&]() -> bool {
+            if (P == ISJL_POLICY_FCFS) return fcfs < rel && run_cnt > 0;
+            return pend > 0 && run_cnt > 0;
+        };
         auto batch = [&]() -> bool {
             if (skip > 0) { skip--; return false; }
             if (nn < 6 && nn < run_cnt) {
@@ -1123,14 +1215,26 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
             }
             // lane i: completion i and the KV it frees
             const int32_t ci = kbase + (int32_t)(nk >> SH);
+            const int32_t c_end = kLpt ? min(evt_base, next_arr) : evt_base;
+            if (__shfl_sync(kFull, ci, 0) >= c_end) return false;
             const int from = (int)(nk >> RB) & 31;
             const uint32_t row_i = nk & RM;
             int F = lane < nn ? S.slot[(int)(row_i << 5) + from].y : 0;
             // lane j: request j of the queue
-            if (hbase != fcfs) load_heads();
-            const int nh = min(31, rel - fcfs);
-            const int e = fcfs + lane;
-            const int oe = (int)(hw >> 16), oc = (int)(hw & 0xFFFFu);
+            const int nh = min(31, kLpt ? pend : rel - fcfs);
+            int q = -1, e, oe, oc;
+            if (kLpt) {
+                q = first_pending_from(hp, nh);
+                e = q >= 0 ? perm[q] : 0;
+                oe = q >= 0 ? osrt[q] : 0;
+                oc = (opaque(flags) & kSlack) && q >= 0 ? otru[e] : oe;
+                if (__popc(__ballot_sync(kFull, q >= 0)) != nh) { broken = true; return false; }
+            } else {
+                if (hbase != fcfs) load_heads();
+                e = fcfs + lane;
+                oe = (int)(hw >> 16);
+                oc = (int)(hw & 0xFFFFu);
+            }
             int Pj = lane < nh ? oe : 1 << 25;
             const int u_i = F;
 #pragma unroll
@@ -1162,15 +1266,14 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
             const int32_t first_i = __shfl_sync(kFull, first, jl);
             const int32_t t_l = __shfl_sync(kFull, t_j, jl);
             const int P_l = __shfl_sync(kFull, Pj, jl);
-            const bool ok = lane < nn && ci < evt_base && Jp < nh && ci <= e_lo &&
-                            (Jp > 0 ? first_i > ci : ci <= e_hi);
+            const bool ok = lane < nn && ci < c_end && Jp < nh && ci <= e_lo && (Jp > 0 ? first_i > ci : ci <= e_hi);
             const unsigned no = ~__ballot_sync(kFull, ok);
             int m = no ? __ffs(no) - 1 : 32;
             if (m < nn && m > 0) {                             // not between completions of one step
                 const int32_t cm = __shfl_sync(kFull, ci, m);
                 if (__shfl_sync(kFull, ci, m - 1) == cm) m = __popc(__ballot_sync(kFull, ci < cm));
             }
-            if (m == 0) { nn = 0; return false; }
+            if (m == 0) return false;
             // the steps before each of the m completions
             int32_t t0_i = __shfl_up_sync(kFull, ci, 1);
             if (lane == 0) t0_i = k;
@@ -1205,14 +1308,16 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
             nn -= m;
             if (lane >= nn) nk = kEmpty;
             if (lane < c) {
-                if (st_out) st_out[e] = t_j;
-                if (co_out) co_out[e] = n_j;
+                const int f = opaque(flags);
+                if (f & kHasStart) st_out[e] = t_j;
+                if (f & kHasCompl) co_out[e] = n_j;
                 sums_l += (uint32_t)t_j;
-                if (trunc) {
+                if (f & kTrunc) {
                     R_l += ((uint32_t)oc * (uint32_t)(oc + 1)) >> 1;
                     tok_l += oc;
                 }
             }
+#pragma unroll 1
             for (int placed = 0; placed < c;) {                // one per lane with a free slot and round
                 const bool f = idle != 0u;
                 const unsigned b = __ballot_sync(kFull, f);
@@ -1232,6 +1337,7 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
                     S.slot[(row << 5) + lane] = make_int2(t, u);
                     near = nc < near_end;
                 }
+#pragma unroll 1
                 for (unsigned nb = __ballot_sync(kFull, near); nb; nb &= nb - 1u) {
                     const uint32_t y = __shfl_sync(kFull, x, __ffs(nb) - 1);
                     if (kbase + (int32_t)(y >> SH) < near_end) join(y);
@@ -1247,24 +1353,35 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
             Tmake = k_new;
             kv_sum += (c > 0 ? used : 0) - freed;
             run_cnt += c - m;
-            fcfs += c;
-            fh = __shfl_sync(kFull, hw, c);
-            load_heads();                                      // for the next pass
+            if (kLpt) {
+                clear_pending(q, lane < c);
+                pend -= c;
+                if (c < nh) {
+                    hp = __shfl_sync(kFull, q, c);
+                    ho = __shfl_sync(kFull, oe, c);
+                    he = __shfl_sync(kFull, e, c);
+                    ht = __shfl_sync(kFull, oc, c);
+                } else {
+                    set_head(bs_next(S, words0, words1, __shfl_sync(kFull, q, 0), lane));
+                }
+            } else {
+                fcfs += c;
+                fh = __shfl_sync(kFull, hw, c);
+                load_heads();                                  // for the next pass
+            }
             stale = true;
             __syncwarp();
             return true;
         };
 
         for (;;) {
-            if (min(e_lo, e_hi) <= k) {
-                if (run_cnt > 0) {
-                    rescan();
-                } else {                                         // nothing runs: the steps up to evt are idle
-                    if (P == ISJL_POLICY_FCFS ? fcfs == n : rel == n && pend == 0 && plan_left == 0) break;
-                    if (evt >= (1 << 30) - 1) { status = ISJL_ERR_INTERNAL; break; }   // cannot progress
-                    smin = smax;
-                    Tb -= evt - k;
-                }
+            if (run_cnt == 0) {                                  // nothing runs: the steps up to evt are idle
+                if (P == ISJL_POLICY_FCFS ? fcfs == n : rel == n && pend == 0 && plan_left == 0) break;
+                if (evt >= (1 << 30) - 1) { status = ISJL_ERR_INTERNAL; break; }   // cannot progress
+                smin = smax;
+                Tb -= evt - k;
+            } else if (!kIsjl && min(e_lo, e_hi) <= k) {
+                rescan();
             }
             bool served = false;
             if (kBatch) served = waits() && batch();
@@ -1325,7 +1442,7 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
                     Tmake = k;
                     nn = 0;
                     do {
-                        pop_front(f, freed);
+                        if (f) pop_front(freed);
                         run_cnt -= __popc(b);
                         f = key0 <= thr;
                         b = __ballot_sync(kFull, f);
@@ -1333,6 +1450,7 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
                     kv_sum -= (int32_t)__reduce_add_sync(kFull, (unsigned)freed);
                 }
             }
+            if (kIsjl && min(e_lo, e_hi) <= k && run_cnt > 0) rescan();   // the gate looks at smin
             // ---- starts
             admit();
             if (broken) { status = ISJL_ERR_INTERNAL; break; }
@@ -1373,9 +1491,11 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
             sumc = sums + (int64_t)__reduce_add_sync(kFull, (unsigned)tok_l) - warp_sum64(run_c);
             if (co_out) {
                 __syncwarp();
+#pragma unroll 1
                 for (int i = lane; i < n; i += 32)
                     if (status != ISJL_ERR_STEP_LIMIT || co_out[i] >= k) co_out[i] = -1;
                 if (st_out && status != ISJL_ERR_STEP_LIMIT)
+#pragma unroll 1
                     for (int i = lane; i < n; i += 32) st_out[i] = -1;
             }
         }
@@ -1451,20 +1571,23 @@ sim_kernel(SimArgs A, int64_t n_tasks) {
     S.slong = b + 3 * A.B;
     S.pend0 = reinterpret_cast<uint32_t *>(b + 4 * A.B);
     S.pend1 = S.pend0 + A.words0;
-    const int64_t gwarp = (int64_t)blockIdx.x * kSimWarpsPerBlock + wib;
+    const int64_t gwarp = (int64_t)blockIdx.x * (blockDim.x >> 5) + wib;
     for (;;) {
         int t = 0;
         if (lane == 0) t = atomicAdd(A.task_counter, 1);
         t = (int)__reduce_max_sync(kFull, (unsigned)t);
         if ((int64_t)t >= n_tasks) break;
         // run-major: at any time the warps of an SM mostly run one policy's code
-        const int64_t inst = t % A.n_inst;
-        const int run = (int)(t / A.n_inst);
+        const int run = (int)((uint32_t)t / (uint32_t)A.n_inst);   // n_inst and the task count are below 2^31
+        const int64_t inst = t - (int64_t)run * A.n_inst;
         switch (A.runs.policy[run]) {
             case ISJL_POLICY_FCFS: run_task<SPL, ISJL_POLICY_FCFS>(A, S, lane, gwarp, inst, run); break;
             case ISJL_POLICY_LJF:  run_task<SPL, ISJL_POLICY_LJF>(A, S, lane, gwarp, inst, run); break;
             case ISJL_POLICY_SJF:  run_task<SPL, ISJL_POLICY_SJF>(A, S, lane, gwarp, inst, run); break;
-            default:               run_task<SPL, ISJL_POLICY_ISJL>(A, S, lane, gwarp, inst, run); break;
+            default:
+                if (A.runs.delta[run] >= ISJL_MAX_LEN) run_task<SPL, kPolicyLpt>(A, S, lane, gwarp, inst, run);
+                else run_task<SPL, ISJL_POLICY_ISJL>(A, S, lane, gwarp, inst, run);
+                break;
         }
     }
 }
@@ -1495,39 +1618,59 @@ size_t sim_smem_per_warp(int B, int n) {
     return (size_t)smem_words_per_warp(slots_per_lane(B), B, words0, words1) * 4;
 }
 
-static cudaError_t occupancy(int B, int n, int device, int *blocks_per_sm, int *sms, size_t *smem) {
+// warps per block and the dynamic shared memory of one (0: n is too large for this B).
+// n is accepted as long as four warps with seven words per slot and the pending
+// bitset would fit; where four warps' actual layout does not, fewer share a block
+static cudaError_t block_shape(int B, int n, int device, int *warps, size_t *smem) {
+    int limit = 0;
+    const cudaError_t e = cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
+    if (e != cudaSuccess) return e;
+    const int64_t words0 = (n + 31) / 32, words1 = (words0 + 31) / 32;
+    const int64_t bound = kSimWarpsPerBlock * (((7 * (int64_t)B + words0 + words1 + 3) & ~(int64_t)3) * 4);
+    const size_t per = sim_smem_per_warp(B, n);
+    *warps = 0;
+    *smem = 0;
+    if (bound > limit) return cudaSuccess;
+    *warps = (int)std::min<size_t>(kSimWarpsPerBlock, (size_t)limit / per);
+    *smem = per * *warps;
+    return cudaSuccess;
+}
+
+static cudaError_t occupancy(int B, int n, int device, int *blocks_per_sm, int *sms, int *warps, size_t *smem) {
+    cudaError_t e = block_shape(B, n, device, warps, smem);
+    if (e != cudaSuccess) return e;
+    if (*warps < 1) return cudaErrorInvalidValue;
     const void *k = pick_kernel(slots_per_lane(B));
-    *smem = sim_smem_per_warp(B, n) * kSimWarpsPerBlock;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*smem);
+    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*smem);
     if (e != cudaSuccess) return e;
     e = cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, device);
     if (e != cudaSuccess) return e;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, kSimWarpsPerBlock * 32, *smem);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, *warps * 32, *smem);
 }
 
 int sim_resident_warps(int B, int n, int device) {
-    int bps = 0, sms = 0;
+    int bps = 0, sms = 0, warps = 0;
     size_t smem = 0;
-    if (occupancy(B, n, device, &bps, &sms, &smem) != cudaSuccess || bps < 1) return 0;
-    return bps * sms * kSimWarpsPerBlock;
+    if (occupancy(B, n, device, &bps, &sms, &warps, &smem) != cudaSuccess || bps < 1) return 0;
+    return bps * sms * warps;
 }
 
 cudaError_t launch_sim(const SimArgs &args, int total_warps, cudaStream_t s) {
-    int bps = 0, sms = 0, dev = 0;
+    int bps = 0, sms = 0, dev = 0, warps = 0;
     size_t smem = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    e = occupancy(args.B, args.n, dev, &bps, &sms, &smem);
+    e = occupancy(args.B, args.n, dev, &bps, &sms, &warps, &smem);
     if (e != cudaSuccess) return e;
     const int64_t n_tasks = args.n_inst * args.n_runs;
-    int64_t blocks = total_warps / kSimWarpsPerBlock;
-    const int64_t need = (n_tasks + kSimWarpsPerBlock - 1) / kSimWarpsPerBlock;
+    int64_t blocks = total_warps / warps;
+    const int64_t need = (n_tasks + warps - 1) / warps;
     if (blocks > need) blocks = need;
     if (blocks < 1) blocks = 1;
     const void *k = pick_kernel(slots_per_lane(args.B));
     SimArgs a = args;
     void *params[] = {&a, const_cast<int64_t *>(&n_tasks)};
-    return cudaLaunchKernel(k, dim3((unsigned)blocks), dim3(kSimWarpsPerBlock * 32), params, smem, s);
+    return cudaLaunchKernel(k, dim3((unsigned)blocks), dim3(warps * 32), params, smem, s);
 }
 
 }  // namespace isjl

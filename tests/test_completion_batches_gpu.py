@@ -10,7 +10,7 @@ from test_parity_gpu import INF, O, S, run_both  # noqa: F401  (fixtures)
 
 pytestmark = [pytest.mark.gpu, pytest.mark.skipif(not cuda_available(), reason="needs a CUDA GPU")]
 
-POLICIES = ["fcfs"]
+POLICIES = ["fcfs", "isjl"]
 
 
 def lengths(rng, kind, shape):
@@ -40,4 +40,4 @@ def test_batches_of_completions(S, O, policy, kind, B):  # noqa: F811
                           (big + 40, rng.integers(0, 40, o.shape).astype(np.int32), 0), (big * 3, None, 997)]:
         if slack is not None:
             o = np.minimum(o, 65_535 - 40)
-        run_both(S, O, a, p, o, B, [policy], [50], kv, False, slack=slack, max_steps=ms)
+        run_both(S, O, a, p, o, B, [policy] * 2, [50, INF], kv, False, slack=slack, max_steps=ms)
