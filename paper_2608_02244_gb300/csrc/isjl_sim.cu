@@ -142,9 +142,7 @@ isjl_status isjl_sim_run_sweep(isjl_sim *s, int32_t n_runs, const int32_t *polic
         runs.beta[i] = isjl::run_beta(policies[i], deltas[i]);
     }
 
-    if (cudaMemsetAsync(s->d_counter, 0, sizeof(int32_t), st) != cudaSuccess ||
-        cudaMemsetAsync(s->d_status, 0, sizeof(int32_t), st) != cudaSuccess || !mark(0))
-        return ISJL_ERR_CUDA;
+    if (!mark(0)) return ISJL_ERR_CUDA;
     if (in->slack && !s->d_otrue && dalloc(&s->d_otrue, s->N) != cudaSuccess) {
         cudaGetLastError();
         s->d_otrue = nullptr;
@@ -152,7 +150,7 @@ isjl_status isjl_sim_run_sweep(isjl_sim *s, int32_t n_runs, const int32_t *polic
     }
     int32_t *otrue = in->slack ? s->d_otrue : nullptr;
     if (isjl::launch_derive(in->arrival, in->prompt, in->output, in->count, in->slack, s->d_o, otrue, s->d_inst,
-                            c.n_instances, c.n_per_instance, st) != cudaSuccess || !mark(1))
+                            s->d_counter, s->d_status, c.n_instances, c.n_per_instance, st) != cudaSuccess || !mark(1))
         return ISJL_ERR_CUDA;
     s->last_launches++;
     if (isjl::launch_sort(s->d_o, s->d_inst, s->d_perm, s->d_osorted, s->d_posof, s->d_tmp, c.n_instances,

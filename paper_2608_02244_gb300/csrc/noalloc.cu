@@ -14,7 +14,7 @@
 // before any stream capture.  Every call uses the same array, so calls whose
 // work overlaps on the GPU (two streams, or two host threads) race and must
 // be serialized by the caller.  The array keeps the previous call's contents:
-// the work counter and status word are zeroed on the stream at each call;
+// the work counter and status word are zeroed by the derive kernel;
 // everything else is written before it is read.
 #include <cstdint>
 #include <cstring>
@@ -105,9 +105,8 @@ extern "C" isjl_status isjl_sim_run_sweep_noalloc(const isjl_config *cfg, int32_
     int32_t *d_plan = reinterpret_cast<int32_t *>(base + plan_off);
 
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (cudaMemsetAsync(d_ctr, 0, 2 * sizeof(int32_t), st) != cudaSuccess) return ISJL_ERR_CUDA;
-    if (isjl::launch_derive(in->arrival, in->prompt, in->output, in->count, in->slack, d_o, d_ot, d_inst,
-                            cfg->n_instances, n, st) != cudaSuccess)
+    if (isjl::launch_derive(in->arrival, in->prompt, in->output, in->count, in->slack, d_o, d_ot, d_inst, d_ctr,
+                            d_ctr + 1, cfg->n_instances, n, st) != cudaSuccess)
         return ISJL_ERR_CUDA;
     if (isjl::launch_sort(d_o, d_inst, d_perm, d_os, d_pos, d_tmp, cfg->n_instances, n, st) != cudaSuccess)
         return ISJL_ERR_CUDA;

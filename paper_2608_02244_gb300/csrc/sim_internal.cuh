@@ -13,7 +13,7 @@ constexpr unsigned kFull = 0xffffffffu;
 constexpr int kWarp = 32;
 constexpr int kSimWarpsPerBlock = 4;         // 128-thread blocks for the simulation kernel
 constexpr int kSortSmallMax = 4096;           // bitonic in shared memory up to this n
-constexpr int kRadixThreads = 128;            // threads of the large-n radix sort
+constexpr int kRadixThreads = 1024;           // threads of the large-n radix sort
 
 // Per-instance facts derived once per call (policy independent).
 struct InstStats {
@@ -58,7 +58,7 @@ struct SimArgs {
     isjl_record *records;      // [n_runs * n_inst]
     int32_t *start_out;        // [n_runs * N] or null
     int32_t *compl_out;        // [n_runs * N] or null
-    int32_t *task_counter;     // work queue head, zeroed before each launch
+    int32_t *task_counter;     // work queue head, zeroed by the derive kernel
     int32_t *dev_status;       // first nonzero status of the launch
     int64_t n_inst;
     int32_t n;
@@ -75,7 +75,8 @@ struct SimArgs {
 // host-side launchers (defined in the .cu files)
 cudaError_t launch_derive(const int32_t *arrival, const int32_t *prompt, const int32_t *output,
                           const int32_t *count, const int32_t *slack, int32_t *o, int32_t *otrue,
-                          InstStats *inst, int64_t n_inst, int32_t n, cudaStream_t s);
+                          InstStats *inst, int32_t *counter, int32_t *dev_status, int64_t n_inst, int32_t n,
+                          cudaStream_t s);
 cudaError_t launch_sort(const int32_t *o, const InstStats *inst, int32_t *perm, int32_t *osorted, int32_t *posof,
                         int32_t *tmp, int64_t n_inst, int32_t n, cudaStream_t s);
 cudaError_t launch_sim(const SimArgs &args, int total_warps, cudaStream_t s);

@@ -10,7 +10,7 @@ from test_parity_gpu import INF, O, S, run_both  # noqa: F401  (fixtures)
 
 pytestmark = [pytest.mark.gpu, pytest.mark.skipif(not cuda_available(), reason="needs a CUDA GPU")]
 
-POLICIES = ["fcfs", "isjl"]
+POLICIES = ["fcfs", "isjl", "sjf"]
 
 
 def lengths(rng, kind, shape):
