@@ -272,6 +272,7 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
     constexpr int32_t kSpan = 1 << (30 - SH);       // kbase follows k when it is this far behind
     constexpr bool kIsjl = P == ISJL_POLICY_ISJL;
     constexpr bool kLpt = P == kPolicyLpt;
+    constexpr bool kSjf = P == ISJL_POLICY_SJF;
     constexpr bool kBatch = P == ISJL_POLICY_FCFS || kLpt;
     const int n_slots = A.n, B = A.B;
     const int64_t base = inst * (int64_t)n_slots;
@@ -368,11 +369,12 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
         int32_t k = -1, kbase = 0, rel = 0, fcfs = 0, run_cnt = 0, pend = 0;
         int32_t kv_sum = 0;
         // the next 32 unreleased requests (from win_base): arrival and sorted position, per lane
-        int32_t win_base = 0, win_a = INT_MAX, win_p = 0;
+        int32_t win_base = 0, win_a = INT_MAX, win_p = 0, win_u = 0;   // (SJF) and planning length
         auto load_window = [&]() {
             const int i = win_base + lane;
             win_a = i < n ? arr[i] : INT_MAX;
             win_p = (i < n && P != ISJL_POLICY_FCFS) ? posof[i] : 0;
+            if (kSjf) win_u = i < n ? oarr[i] : INT_MAX;
         };
         load_window();
         // FCFS: lengths (planning above true) of the 32 requests from hbase on, per
@@ -397,6 +399,7 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
         // LJF / ISJL: the longest pending position, SJF: the last one (of the
         // shortest length), with its planning length, index and true length
         int32_t hp = P == ISJL_POLICY_SJF ? -1 : INT_MAX, ho = 0, he = 0, ht = 0;
+        bool h_tie = false;                            // SJF: the position before it has the same length
         // start range of the running set and the last completions of those started
         // at its ends; found again (rescan) once e_lo or e_hi is reached
         int32_t smin = 0, smax = 0, e_lo = INT_MIN, e_hi = INT_MIN;
@@ -559,6 +562,7 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
             hp = p;
             if (p >= 0 && p < n) {
                 ho = osrt[p];
+                if (kSjf) h_tie = p > 0 && osrt[p - 1] == ho;
                 he = perm[p];
                 ht = (opaque(flags) & kSlack) ? otru[he] : ho;
             }
@@ -619,6 +623,19 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
             __syncwarp();
             pend--;
             set_head(v ? (w << 5) + __ffs(v) - 1 : bs_next(S, words0, words1, (w + 1) << 5, lane));
+        };
+        // SJF: remove the last pending position, hp (nothing is pending above it)
+        auto pop_tail = [&]() {
+            const int w = hp >> 5;
+            const uint32_t v = S.pend0[w] & ~(1u << (hp & 31));
+            __syncwarp();
+            if (lane == 0) {
+                S.pend0[w] = v;
+                if (!v) S.pend1[w >> 5] &= ~(1u << (w & 31));
+            }
+            __syncwarp();
+            pend--;
+            set_head(v ? (w << 5) + 31 - __clz(v) : bs_prev(S, (w << 5) - 1, lane));
         };
         // sorted positions of the first m (1 <= m <= 32) pending requests at or
         // after position p0: lane l gets the l-th, lanes past the last one -1
@@ -953,13 +970,14 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
         // After an admission, `blocked` says that no arrival alone can let a
         // request start before the next completion (or o_1's delay expiry):
         // FCFS with B full or its head not fitting the KV cap, LJF with a batch
-        // running, SJF with B full, ISJL with its gate closed or its queue
+        // running, SJF with B full or no arrival that fits, ISJL with its gate closed or its queue
         // stopped on the KV cap or on workers (an arrival never becomes a head
         // that fits better: it sorts after every pending request of its length).
         // Arrivals are then released at the next event instead of ending the
         // interval there.
         auto admit = [&]() {
             bool blocked;
+            int32_t next_fit = INT_MAX;
             if (P == ISJL_POLICY_FCFS) {
                 // arrival order; the first request that does not fit ends the step;
                 // one at a time for the first two starts (usually all there are),
@@ -987,6 +1005,11 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
 #pragma unroll 1
                 for (int nseq = 0; pend > 0 && kv_sum + ho <= kv_lim && run_cnt < B; ++nseq) {
                     if (hp < 0 || hp >= n) { broken = true; return; }
+                    if (!h_tie && nseq < 2) {                    // the only position of its length
+                        start_any(he, ho, ht, idle, __ballot_sync(kFull, idle != 0u));
+                        pop_tail();
+                        continue;
+                    }
                     // first position of this length: usually among the 32 up to hp
                     const int i = hp - lane;
                     const unsigned other = __ballot_sync(kFull, i < 0 || osrt[max(i, 0)] != ho);
@@ -1010,7 +1033,14 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
                         set_head(bs_prev(S, hp, lane));
                     }
                 }
-                blocked = run_cnt >= B;
+                // what waits does not fit, and nor do the arrivals longer than the KV
+                // left: the next that fits, or past this window the window's last
+                if (run_cnt < B && rel < n) {
+                    const int i = win_base + lane;
+                    const unsigned b = __ballot_sync(kFull, i >= rel && (win_u <= kv_lim - kv_sum || (lane == 31 && i < n)));
+                    next_fit = b ? __shfl_sync(kFull, win_a, __ffs(b) - 1) : INT_MAX;
+                }
+                blocked = run_cnt >= B || next_fit == INT_MAX;
             } else if (P == ISJL_POLICY_LJF) {
                 // static batch of the longest released requests when nothing runs
                 if (run_cnt == 0) start_longest();
@@ -1062,7 +1092,7 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
                 if (!stop) start_longest();   // Phase TWO: longest released first
                 blocked = stop || pend > 0;
             }
-            evt = blocked && run_cnt > 0 ? evt_base : min(evt_base, next_arr);
+            evt = blocked && run_cnt > 0 ? evt_base : min(evt_base, kSjf ? next_fit : next_arr);
             if (kIsjl && !L1_started && t0 + d1 > k) evt = min(evt, t0 + d1);
         };
 
