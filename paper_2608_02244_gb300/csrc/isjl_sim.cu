@@ -18,7 +18,7 @@ struct isjl_sim {
     int32_t *d_otrue = nullptr;      // true lengths, allocated on the first call with slack
     InstStats *d_inst = nullptr;
     int32_t *d_plan_next = nullptr;
-    int total_warps = 0;
+    isjl::SimShape shape{0, 0, 0};
     int32_t *d_counter = nullptr, *d_status = nullptr;
     isjl_summary *d_summary = nullptr;
     // buffers of the host-memory entry point, allocated on first use
@@ -94,12 +94,11 @@ isjl_status isjl_sim_create(const isjl_config *cfg, isjl_sim **out) {
     s->N = cfg->n_instances * (int64_t)cfg->n_per_instance;
     if (cudaGetDevice(&s->device) != cudaSuccess) { delete s; return ISJL_ERR_CUDA; }
     const int n = cfg->n_per_instance;
-    s->total_warps = isjl::sim_resident_warps(cfg->B, n, s->device);
-    if (s->total_warps < 1) { delete s; cudaGetLastError(); return ISJL_ERR_INVALID_ARG; }   // B, n too large for smem
+    if (isjl::sim_shape(cfg->B, n, s->device, &s->shape) != cudaSuccess || s->shape.warps < 1) { delete s; cudaGetLastError(); return ISJL_ERR_INVALID_ARG; }   // B, n too large for smem
     bool ok = dalloc(&s->d_o, s->N) == cudaSuccess && dalloc(&s->d_perm, s->N) == cudaSuccess &&
               dalloc(&s->d_osorted, s->N) == cudaSuccess && dalloc(&s->d_posof, s->N) == cudaSuccess &&
               dalloc(&s->d_inst, cfg->n_instances) == cudaSuccess &&
-              dalloc(&s->d_plan_next, (size_t)s->total_warps * n) == cudaSuccess &&
+              dalloc(&s->d_plan_next, (size_t)s->shape.warps * n) == cudaSuccess &&
               dalloc(&s->d_counter, 1) == cudaSuccess && dalloc(&s->d_status, 1) == cudaSuccess &&
               dalloc(&s->d_summary, ISJL_MAX_RUNS) == cudaSuccess;
     if (ok && n > isjl::kSortSmallMax) ok = dalloc(&s->d_tmp, s->N) == cudaSuccess;
@@ -134,13 +133,7 @@ isjl_status isjl_sim_run_sweep(isjl_sim *s, int32_t n_runs, const int32_t *polic
     s->timed = false;
     const bool timing = (c.flags & ISJL_FLAG_TIMING) != 0u;
     auto mark = [&](int i) { return !timing || cudaEventRecord(s->ev[i], st) == cudaSuccess; };
-    RunList runs;
-    std::memset(&runs, 0, sizeof(runs));
-    for (int i = 0; i < n_runs; ++i) {
-        runs.policy[i] = policies[i];
-        runs.delta[i] = deltas[i];
-        runs.beta[i] = isjl::run_beta(policies[i], deltas[i]);
-    }
+    const RunList runs = isjl::run_list(n_runs, policies, deltas);
 
     if (!mark(0)) return ISJL_ERR_CUDA;
     if (in->slack && !s->d_otrue && dalloc(&s->d_otrue, s->N) != cudaSuccess) {
@@ -185,7 +178,7 @@ isjl_status isjl_sim_run_sweep(isjl_sim *s, int32_t n_runs, const int32_t *polic
     a.tau = c.tau;
     a.p0 = c.p0;
     a.runs = runs;
-    if (isjl::launch_sim(a, s->total_warps, st) != cudaSuccess || !mark(3)) return ISJL_ERR_CUDA;
+    if (isjl::launch_sim(a, s->shape, st) != cudaSuccess || !mark(3)) return ISJL_ERR_CUDA;
     s->last_launches++;
     if (isjl::launch_summarize(out->records, c.n_instances, n_runs, runs, kv_cap, s->d_summary, st) !=
             cudaSuccess || !mark(4))

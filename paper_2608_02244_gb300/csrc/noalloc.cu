@@ -86,11 +86,11 @@ extern "C" isjl_status isjl_sim_run_sweep_noalloc(const isjl_config *cfg, int32_
     if (off >= kScratchBytes) return ISJL_ERR_INVALID_ARG;   // too large for the fixed workspace
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return ISJL_ERR_CUDA;
-    int warps = isjl::sim_resident_warps(cfg->B, n, dev);
-    if (warps < 1) return ISJL_ERR_INVALID_ARG;
+    isjl::SimShape shape;
+    if (isjl::sim_shape(cfg->B, n, dev, &shape) != cudaSuccess || shape.warps < 1) return ISJL_ERR_INVALID_ARG;
     const int64_t fit = (int64_t)((kScratchBytes - plan_off) / (sizeof(int32_t) * (size_t)n));
-    if (fit < warps) warps = (int)(fit / isjl::kSimWarpsPerBlock) * isjl::kSimWarpsPerBlock;
-    if (warps < isjl::kSimWarpsPerBlock) return ISJL_ERR_INVALID_ARG;   // plan scratch for one block does not fit
+    if (fit < shape.warps) shape.warps = (int)(fit / isjl::kSimWarpsPerBlock) * isjl::kSimWarpsPerBlock;
+    if (shape.warps < isjl::kSimWarpsPerBlock) return ISJL_ERR_INVALID_ARG;   // plan scratch for four warps does not fit
 
     unsigned char *base = nullptr;
     if (scratch_ptr(&base) != cudaSuccess) return ISJL_ERR_CUDA;
@@ -137,11 +137,7 @@ extern "C" isjl_status isjl_sim_run_sweep_noalloc(const isjl_config *cfg, int32_
     a.c = cfg->c;
     a.tau = cfg->tau;
     a.p0 = cfg->p0;
-    for (int i = 0; i < n_runs; ++i) {
-        a.runs.policy[i] = policies[i];
-        a.runs.delta[i] = deltas[i];
-        a.runs.beta[i] = isjl::run_beta(policies[i], deltas[i]);
-    }
-    if (isjl::launch_sim(a, warps, st) != cudaSuccess) return ISJL_ERR_CUDA;
+    a.runs = isjl::run_list(n_runs, policies, deltas);
+    if (isjl::launch_sim(a, shape, st) != cudaSuccess) return ISJL_ERR_CUDA;
     return ISJL_OK;
 }

@@ -1607,9 +1607,11 @@ sim_kernel(SimArgs A, int64_t n_tasks) {
         if (lane == 0) t = atomicAdd(A.task_counter, 1);
         t = (int)__reduce_max_sync(kFull, (unsigned)t);
         if ((int64_t)t >= n_tasks) break;
-        // run-major: at any time the warps of an SM mostly run one policy's code
-        const int run = (int)((uint32_t)t / (uint32_t)A.n_inst);   // n_inst and the task count are below 2^31
-        const int64_t inst = t - (int64_t)run * A.n_inst;
+        // run-major: at any time the warps of an SM mostly run one policy's code;
+        // the runs with the longest tasks first, so that short tasks fill the tail
+        const int turn = (int)((uint32_t)t / (uint32_t)A.n_inst);   // n_inst and the task count are below 2^31
+        const int64_t inst = t - (int64_t)turn * A.n_inst;
+        const int run = A.runs.order[turn];
         switch (A.runs.policy[run]) {
             case ISJL_POLICY_FCFS: run_task<SPL, ISJL_POLICY_FCFS>(A, S, lane, gwarp, inst, run); break;
             case ISJL_POLICY_LJF:  run_task<SPL, ISJL_POLICY_LJF>(A, S, lane, gwarp, inst, run); break;
@@ -1666,41 +1668,35 @@ static cudaError_t block_shape(int B, int n, int device, int *warps, size_t *sme
     return cudaSuccess;
 }
 
-static cudaError_t occupancy(int B, int n, int device, int *blocks_per_sm, int *sms, int *warps, size_t *smem) {
-    cudaError_t e = block_shape(B, n, device, warps, smem);
-    if (e != cudaSuccess) return e;
-    if (*warps < 1) return cudaErrorInvalidValue;
+cudaError_t sim_shape(int B, int n, int device, SimShape *out) {
+    *out = SimShape{0, 0, 0};
+    cudaError_t e = block_shape(B, n, device, &out->warps_per_block, &out->smem);
+    if (e != cudaSuccess || out->warps_per_block < 1) return e;
     const void *k = pick_kernel(slots_per_lane(B));
-    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*smem);
+    // the same for every caller, so that no other shape's use of the kernel changes it
+    int limit = 0, bps = 0, sms = 0;
+    e = cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
     if (e != cudaSuccess) return e;
-    e = cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, device);
+    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, limit);
     if (e != cudaSuccess) return e;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, *warps * 32, *smem);
+    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
+    if (e != cudaSuccess) return e;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k, out->warps_per_block * 32, out->smem);
+    if (e != cudaSuccess) return e;
+    out->warps = bps * sms * out->warps_per_block;
+    return cudaSuccess;
 }
 
-int sim_resident_warps(int B, int n, int device) {
-    int bps = 0, sms = 0, warps = 0;
-    size_t smem = 0;
-    if (occupancy(B, n, device, &bps, &sms, &warps, &smem) != cudaSuccess || bps < 1) return 0;
-    return bps * sms * warps;
-}
-
-cudaError_t launch_sim(const SimArgs &args, int total_warps, cudaStream_t s) {
-    int bps = 0, sms = 0, dev = 0, warps = 0;
-    size_t smem = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    e = occupancy(args.B, args.n, dev, &bps, &sms, &warps, &smem);
-    if (e != cudaSuccess) return e;
-    const int64_t n_tasks = args.n_inst * args.n_runs;
-    int64_t blocks = total_warps / warps;
-    const int64_t need = (n_tasks + warps - 1) / warps;
+cudaError_t launch_sim(const SimArgs &args, const SimShape &shape, cudaStream_t s) {
+    const int64_t n_tasks = args.n_inst * args.n_runs, per = shape.warps_per_block;
+    int64_t blocks = shape.warps / per;
+    const int64_t need = (n_tasks + per - 1) / per;
     if (blocks > need) blocks = need;
     if (blocks < 1) blocks = 1;
     const void *k = pick_kernel(slots_per_lane(args.B));
     SimArgs a = args;
     void *params[] = {&a, const_cast<int64_t *>(&n_tasks)};
-    return cudaLaunchKernel(k, dim3((unsigned)blocks), dim3(warps * 32), params, smem, s);
+    return cudaLaunchKernel(k, dim3((unsigned)blocks), dim3((unsigned)per * 32), params, shape.smem, s);
 }
 
 }  // namespace isjl

@@ -293,10 +293,7 @@ class Simulator:
     def sweep_async(self, arrival, prompt, output, policies, deltas, kv_cap, per_request=False, stream=None,
                     counts=None, slack=None):
         """Launch a sweep on device-resident int32 tensors; returns output tensors."""
-        rec, st, co = self.buffers(len(policies), per_request)
-        if per_request:
-            st.fill_(-1)
-            co.fill_(-1)
+        rec, st, co = self.buffers(len(policies), per_request)   # the kernels write every entry
         _check(isjl_sim_run_sweep(self.handle, policies, deltas, kv_cap, arrival, prompt, output, rec, st, co,
                                   stream, counts, slack), "isjl_sim_run_sweep")
         return rec, st, co
