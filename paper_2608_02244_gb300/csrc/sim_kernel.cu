@@ -301,7 +301,10 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
     if (status == ISJL_OK && is.maxo > kv_lim) status = ISJL_ERR_INFEASIBLE;
     // every schedule ends by sum o + max arrival; completion steps need < 2^30
     if (status == ISJL_OK && is.O + (int64_t)is.maxA + 1 >= (int64_t)(1 << 30)) status = ISJL_ERR_INVALID_ARG;
-    const bool trunc = A.max_steps > 0;             // the run may be stopped early
+    // the run may stop early: at the caller's max_steps, or with predictions at the
+    // step bound, which holds for exact lengths (a pack that finishes before its
+    // planned time leaves o_1's delay idle)
+    const bool trunc = A.max_steps > 0 || otru != nullptr;
     // conditions of the whole task, tested through opaque()
     const int kHasStart = 1, kHasCompl = 2, kTrunc = 4, kSlack = 8, kPacked = 16;
     const int flags = (st_out ? kHasStart : 0) | (co_out ? kHasCompl : 0) | (trunc ? kTrunc : 0) |
@@ -421,7 +424,7 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
         int32_t plan_left = 0, t0 = 0, d1 = 0, nlong = 0;
         bool L1_started = true;
         bool broken = false;   // an internal invariant failed: stop without touching memory
-        const int64_t max_steps = trunc ? A.max_steps : (is.O + (int64_t)is.maxA + 1);
+        const int64_t max_steps = A.max_steps > 0 ? A.max_steps : is.O + (int64_t)is.maxA + 1;
         const int32_t step_guard = (int32_t)min(max_steps + 1, (int64_t)INT_MAX);
         // the next step at which something other than a completion happens: the
         // guard, a new kbase, an arrival or o_1's delay expiry
