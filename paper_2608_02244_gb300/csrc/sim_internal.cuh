@@ -107,6 +107,60 @@ struct SimArgs {
     RunList runs;
 };
 
+// status of a task before it runs: the instance's, an infeasible length or an
+// instance beyond the step counter's range (every schedule ends by sum o + max
+// arrival; completion steps need < 2^30)
+__device__ __forceinline__ int64_t task_status(const InstStats &is, int32_t kv_lim) {
+    if (is.status != ISJL_OK) return is.status;
+    if (is.maxo > kv_lim) return ISJL_ERR_INFEASIBLE;
+    return is.O + (int64_t)is.maxA + 1 >= (int64_t)(1 << 30) ? ISJL_ERR_INVALID_ARG : ISJL_OK;
+}
+
+// what a simulation kernel counted for one task
+struct RecordTotals {
+    int64_t W, E, sum_completion, sum_extent;
+    int32_t T_make, T_busy, token_adv, max_extent, violations, peak_kv, peak_batch;
+    int64_t status;
+};
+
+// one thread writes the task's record
+__device__ __forceinline__ void store_record(const SimArgs &A, const InstStats &is, int64_t inst, int run,
+                                             const RecordTotals &t) {
+    isjl_record R;
+    const bool bad_input = t.status == ISJL_ERR_INVALID_ARG || t.status == ISJL_ERR_INFEASIBLE;
+    R.T_make = bad_input ? 0 : t.T_make;
+    R.T_busy = bad_input ? 0 : t.T_busy;
+    R.O = bad_input ? 0 : is.O;
+    R.Q = bad_input ? 0 : is.Q;
+    R.W = t.W;
+    R.E = t.E;
+    R.token_adv = t.token_adv;
+    R.sum_completion = t.sum_completion;
+    R.sum_latency = bad_input ? 0 : t.sum_completion - is.sumA;
+    R.sum_extent = t.sum_extent;
+    R.max_extent = t.max_extent;
+    R.violations = t.violations;
+    R.kv_violations = 0;   // every start keeps the reservation within the cap
+    R.peak_kv = t.peak_kv;
+    R.peak_batch = t.peak_batch;
+    R.status = t.status;
+    if (bad_input) {
+        R.c_T = R.tau_Q = R.tau_E = R.cost = R.revenue = R.profit = R.throughput = R.ael = 0.0;
+    } else {
+        // cost decomposition C = tau Q + c T + tau E, no contraction
+        R.c_T = __dmul_rn(A.c, (double)t.T_busy);
+        R.tau_Q = __dmul_rn(A.tau, (double)is.Q);
+        R.tau_E = __dmul_rn(A.tau, (double)t.E);
+        R.cost = __dadd_rn(__dadd_rn(R.c_T, R.tau_Q), R.tau_E);
+        R.revenue = __dmul_rn(A.p0, (double)is.O);
+        R.profit = __dsub_rn(R.revenue, R.cost);
+        R.throughput = t.T_make > 0 ? __ddiv_rn((double)is.O, (double)t.T_make) : 0.0;
+        R.ael = is.n > 0 ? __ddiv_rn((double)t.sum_completion, (double)is.n) : 0.0;
+    }
+    A.records[(int64_t)run * A.n_inst + inst] = R;
+    if (t.status != ISJL_OK) atomicCAS(A.dev_status, 0, (int32_t)t.status);
+}
+
 // host-side launchers (defined in the .cu files)
 cudaError_t launch_derive(const int32_t *arrival, const int32_t *prompt, const int32_t *output,
                           const int32_t *count, const int32_t *slack, int32_t *o, int32_t *otrue,
@@ -116,6 +170,9 @@ cudaError_t launch_sort(const int32_t *o, const InstStats *inst, int32_t *perm, 
                         int32_t *tmp, int64_t n_inst, int32_t n, cudaStream_t s);
 cudaError_t sim_shape(int B, int n, int device, SimShape *out);
 cudaError_t launch_sim(const SimArgs &args, const SimShape &shape, cudaStream_t s);
+// instances of at most kTinyMax requests, one thread per task
+constexpr int kTinyMax = 32;
+cudaError_t launch_tiny(const SimArgs &args, cudaStream_t s);
 cudaError_t launch_summarize(const isjl_record *records, int64_t n_inst, int32_t n_runs,
                              const RunList &runs, int32_t kv_cap, isjl_summary *out, cudaStream_t s);
 size_t sim_smem_per_warp(int B, int n);

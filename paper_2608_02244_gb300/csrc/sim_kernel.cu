@@ -297,10 +297,7 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
     int32_t *co_out = A.compl_out ? A.compl_out + out_off : nullptr;
     const int words0 = (n + 31) >> 5, words1 = (words0 + 31) >> 5;
 
-    int64_t status = is.status;
-    if (status == ISJL_OK && is.maxo > kv_lim) status = ISJL_ERR_INFEASIBLE;
-    // every schedule ends by sum o + max arrival; completion steps need < 2^30
-    if (status == ISJL_OK && is.O + (int64_t)is.maxA + 1 >= (int64_t)(1 << 30)) status = ISJL_ERR_INVALID_ARG;
+    int64_t status = task_status(is, kv_lim);
     // the run may stop early: at the caller's max_steps, or with predictions at the
     // step bound, which holds for exact lengths (a pack that finishes before its
     // planned time leaves o_1's delay idle)
@@ -1546,41 +1543,8 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
         }
     }
 
-    if (lane == 0) {
-        isjl_record R;
-        const bool bad_input = status == ISJL_ERR_INVALID_ARG || status == ISJL_ERR_INFEASIBLE;
-        R.T_make = bad_input ? 0 : Tmake;
-        R.T_busy = bad_input ? 0 : Tb;
-        R.O = bad_input ? 0 : is.O;
-        R.Q = bad_input ? 0 : is.Q;
-        R.W = W;
-        R.E = E;
-        R.token_adv = tok;
-        R.sum_completion = sumc;
-        R.sum_latency = bad_input ? 0 : sumc - is.sumA;
-        R.sum_extent = sumext;
-        R.max_extent = maxext;
-        R.violations = viol;
-        R.kv_violations = 0;   // every start keeps the reservation within the cap
-        R.peak_kv = peakkv;
-        R.peak_batch = peakb;
-        R.status = status;
-        if (bad_input) {
-            R.c_T = R.tau_Q = R.tau_E = R.cost = R.revenue = R.profit = R.throughput = R.ael = 0.0;
-        } else {
-            // cost decomposition C = tau Q + c T + tau E, no contraction
-            R.c_T = __dmul_rn(A.c, (double)Tb);
-            R.tau_Q = __dmul_rn(A.tau, (double)is.Q);
-            R.tau_E = __dmul_rn(A.tau, (double)E);
-            R.cost = __dadd_rn(__dadd_rn(R.c_T, R.tau_Q), R.tau_E);
-            R.revenue = __dmul_rn(A.p0, (double)is.O);
-            R.profit = __dsub_rn(R.revenue, R.cost);
-            R.throughput = Tmake > 0 ? __ddiv_rn((double)is.O, (double)Tmake) : 0.0;
-            R.ael = n > 0 ? __ddiv_rn((double)sumc, (double)n) : 0.0;
-        }
-        A.records[(int64_t)run * A.n_inst + inst] = R;
-        if (status != ISJL_OK) atomicCAS(A.dev_status, 0, (int32_t)status);
-    }
+    if (lane == 0)
+        store_record(A, is, inst, run, RecordTotals{W, E, sumc, sumext, Tmake, Tb, tok, maxext, viol, peakkv, peakb, status});
     __syncwarp();
 }
 
@@ -1704,6 +1668,13 @@ cudaError_t sim_shape(int B, int n, int device, SimShape *out) {
 
 cudaError_t launch_sim(const SimArgs &args, const SimShape &shape, cudaStream_t s) {
     const int64_t n_tasks = args.n_inst * args.n_runs, per = shape.warps_per_block;
+    // A thread takes longer over a task than a warp, the more so the more requests n
+    // and workers w = min(B, n) it has, but all threads run at once.  Measured, the
+    // thread per task is faster from about 1 + n (16 + w) / 160 waves of resident
+    // warps on: n = 6 2 waves, n = 12 2 to 4, n = 20 2 to 6.5, n = 32 3 (w = 3), 5
+    // (8), 10 (32); below it is up to 4 times slower
+    const int64_t w = std::min(args.B, args.n);
+    if (args.n <= kTinyMax && n_tasks * 160 > shape.warps * (160 + args.n * (16 + w))) return launch_tiny(args, s);
     int64_t blocks = shape.warps / per;
     const int64_t need = (n_tasks + per - 1) / per;
     if (blocks > need) blocks = need;
