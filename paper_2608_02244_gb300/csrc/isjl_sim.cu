@@ -19,7 +19,11 @@ struct isjl_sim {
     InstStats *d_inst = nullptr;
     int32_t *d_plan_next = nullptr;
     isjl::SimShape shape{0, 0, 0};
-    int32_t *d_counter = nullptr, *d_status = nullptr;
+    int32_t *d_counter = nullptr;
+    // one allocation, so that isjl_sim_metrics needs one copy: the device status in
+    // the first kReportHead bytes, then the summaries
+    unsigned char *d_report = nullptr;
+    int32_t *d_status = nullptr;
     isjl_summary *d_summary = nullptr;
     // buffers of the host-memory entry point, allocated on first use
     int32_t *d_in[3] = {nullptr, nullptr, nullptr};
@@ -37,6 +41,8 @@ struct isjl_sim {
 
 namespace {
 
+constexpr size_t kReportHead = 16;
+
 template <typename T>
 cudaError_t dalloc(T **p, size_t count) {
     return cudaMalloc(reinterpret_cast<void **>(p), count * sizeof(T) + 16);
@@ -46,7 +52,7 @@ void free_all(isjl_sim *s) {
     for (cudaEvent_t &e : s->ev)
         if (e) { cudaEventDestroy(e); e = nullptr; }
     void *ptrs[] = {s->d_o, s->d_otrue, s->d_perm, s->d_osorted, s->d_posof, s->d_tmp, s->d_inst, s->d_plan_next,
-                    s->d_counter, s->d_status, s->d_summary, s->d_in[0], s->d_in[1], s->d_in[2], s->d_rec_io,
+                    s->d_counter, s->d_report, s->d_in[0], s->d_in[1], s->d_in[2], s->d_rec_io,
                     s->d_cnt_in, s->d_slack_in};
     for (void *p : ptrs)
         if (p) cudaFree(p);
@@ -99,8 +105,10 @@ isjl_status isjl_sim_create(const isjl_config *cfg, isjl_sim **out) {
               dalloc(&s->d_osorted, s->N) == cudaSuccess && dalloc(&s->d_posof, s->N) == cudaSuccess &&
               dalloc(&s->d_inst, cfg->n_instances) == cudaSuccess &&
               dalloc(&s->d_plan_next, (size_t)s->shape.warps * n) == cudaSuccess &&
-              dalloc(&s->d_counter, 1) == cudaSuccess && dalloc(&s->d_status, 1) == cudaSuccess &&
-              dalloc(&s->d_summary, ISJL_MAX_RUNS) == cudaSuccess;
+              dalloc(&s->d_counter, 1) == cudaSuccess &&
+              dalloc(&s->d_report, kReportHead + ISJL_MAX_RUNS * sizeof(isjl_summary)) == cudaSuccess;
+    s->d_status = reinterpret_cast<int32_t *>(s->d_report);
+    s->d_summary = ok ? reinterpret_cast<isjl_summary *>(s->d_report + kReportHead) : nullptr;
     if (ok && n > isjl::kSortSmallMax) ok = dalloc(&s->d_tmp, s->N) == cudaSuccess;
     if (ok && (cfg->flags & ISJL_FLAG_TIMING))
         for (cudaEvent_t &e : s->ev) ok = ok && cudaEventCreate(&e) == cudaSuccess;
@@ -202,10 +210,13 @@ isjl_status isjl_sim_metrics(isjl_sim *s, isjl_summary *out, int32_t max_runs) {
     if (!s->ran) return ISJL_ERR_NOT_READY;
     if (max_runs < s->last_runs) return ISJL_ERR_INVALID_ARG;
     if (cudaStreamSynchronize(s->last_stream) != cudaSuccess) return ISJL_ERR_CUDA;
-    int32_t dev_status = 0;
-    if (cudaMemcpy(out, s->d_summary, sizeof(isjl_summary) * s->last_runs, cudaMemcpyDeviceToHost) != cudaSuccess ||
-        cudaMemcpy(&dev_status, s->d_status, sizeof(int32_t), cudaMemcpyDeviceToHost) != cudaSuccess)
+    unsigned char report[kReportHead + ISJL_MAX_RUNS * sizeof(isjl_summary)];
+    const size_t bytes = sizeof(isjl_summary) * (size_t)s->last_runs;
+    if (cudaMemcpy(report, s->d_report, kReportHead + bytes, cudaMemcpyDeviceToHost) != cudaSuccess)
         return ISJL_ERR_CUDA;
+    int32_t dev_status = 0;
+    std::memcpy(&dev_status, report, sizeof(dev_status));
+    std::memcpy(out, report + kReportHead, bytes);
     return (isjl_status)dev_status;
 }
 

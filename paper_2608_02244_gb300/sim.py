@@ -25,6 +25,10 @@ KV_INF = 2**31 - 1
 MAX_B, MAX_LEN, MAX_RUNS = 512, 65535, 32
 FLAG_STEP_KERNEL, FLAG_EPOCH_KERNEL, FLAG_TIMING = 0, 1, 2
 
+# inputs of at most this many int32 in all go to the device in one copy: a copy
+# costs about 12 us of host time, packing them about 1 us per 10,000 values
+ONE_COPY_MAX = 1 << 17
+
 _I64 = ["T_make", "T_busy", "O", "Q", "W", "E", "token_adv", "sum_completion", "sum_latency",
         "sum_extent", "max_extent", "violations", "kv_violations", "peak_kv", "peak_batch", "status"]
 _F64 = ["c_T", "tau_Q", "tau_E", "cost", "revenue", "profit", "throughput", "ael"]
@@ -261,8 +265,7 @@ class Simulator:
         self.n_inst, self.n, self.B = int(n_instances), int(n_per_instance), int(B)
         flags = (FLAG_EPOCH_KERNEL if epoch else FLAG_STEP_KERNEL) | (FLAG_TIMING if timing else 0)
         self.handle = isjl_sim_create(n_instances, n_per_instance, B, c, tau, p0, max_steps, flags)
-        self._records = None
-        self._per_req = None
+        self._block = None
 
     def close(self):
         if self.handle:
@@ -276,19 +279,18 @@ class Simulator:
             pass
 
     def buffers(self, n_runs, per_request):
+        """Output tensors, views of one block kept between calls: records, then
+        start and completion steps."""
         torch = self.torch
         need = n_runs * self.n_inst * RECORD_DTYPE.itemsize
-        if self._records is None or self._records.numel() < need:
-            self._records = torch.empty(need, dtype=torch.uint8, device="cuda")
-        rec = self._records[:need]
-        st = co = None
-        if per_request:
-            npr = n_runs * self.n_inst * self.n
-            if self._per_req is None or self._per_req[0].numel() < npr:
-                self._per_req = (torch.empty(npr, dtype=torch.int32, device="cuda"),
-                                 torch.empty(npr, dtype=torch.int32, device="cuda"))
-            st, co = self._per_req[0][:npr], self._per_req[1][:npr]
-        return rec, st, co
+        per = 4 * n_runs * self.n_inst * self.n if per_request else 0
+        if self._block is None or self._block.numel() < need + 2 * per:
+            self._block = torch.empty(need + 2 * per, dtype=torch.uint8, device="cuda")
+        rec = self._block[:need]
+        if not per_request:
+            return rec, None, None
+        return (rec, self._block[need:need + per].view(torch.int32),
+                self._block[need + per:need + 2 * per].view(torch.int32))
 
     def sweep_async(self, arrival, prompt, output, policies, deltas, kv_cap, per_request=False, stream=None,
                     counts=None, slack=None):
@@ -308,19 +310,28 @@ class Simulator:
             t = torch.as_tensor(np.ascontiguousarray(x, dtype=np.int32)) if not torch.is_tensor(x) else x
             return t.to(device="cuda", dtype=torch.int32).contiguous()
 
-        a, p, o = dev(arrival), dev(prompt), dev(output)
-        cnt = dev(counts) if counts is not None else None
-        sl = dev(slack) if slack is not None else None
+        given = [x for x in (arrival, prompt, output, counts, slack) if x is not None]
+        if all(isinstance(x, np.ndarray) for x in given) and sum(x.size for x in given) <= ONE_COPY_MAX:
+            flat = np.concatenate([np.asarray(x, dtype=np.int32).ravel() for x in given])
+            parts = iter(torch.from_numpy(flat).to("cuda").split([x.size for x in given]))
+        else:
+            parts = iter([dev(x) for x in given])
+        a, p, o = next(parts), next(parts), next(parts)
+        cnt = next(parts) if counts is not None else None
+        sl = next(parts) if slack is not None else None
         rec, st, co = self.sweep_async(a, p, o, policies, deltas, kv_cap, per_request, stream, cnt, sl)
         status, summ = isjl_sim_metrics(self.handle)
         R = len(policies)
         out = {
-            "records": records_to_numpy(rec, R, self.n_inst),
+            "records": None,
             "summaries": [summary_to_dict(summ[i]) for i in range(R)],
             "status": status,
             "launches": isjl_sim_last_launches(self.handle),
         }
+        total = rec.numel() + (8 * st.numel() if per_request else 0)
+        host = self._block[:total].cpu().numpy()          # the outputs lie together: one copy
+        out["records"] = host[:rec.numel()].view(RECORD_DTYPE).reshape(R, self.n_inst)
         if per_request:
-            out["start"] = st.cpu().numpy().reshape(R, self.n_inst, self.n)
-            out["completion"] = co.cpu().numpy().reshape(R, self.n_inst, self.n)
+            steps = host[rec.numel():].view(np.int32).reshape(2, R, self.n_inst, self.n)
+            out["start"], out["completion"] = steps[0], steps[1]
         return out
