@@ -12,7 +12,7 @@ is nonempty; value = sum over (instance, run) of T_busy per second.
 --workload picks another workload's run grid (GRIDS below) for the same
 measurement; the default line is the online delta-sweep.
 
-  python bench.py [--gpus N] [--steps K] [--warmup W] [--kernel step|epoch] [--workload 3|4|5|6|8]
+  python bench.py [--gpus N] [--steps K] [--warmup W] [--workload 1|2|3|4|5|6|8]
   python bench.py --impl reference ...     (the CPU oracle on host cores)
 
 Multi-GPU (torchrun): rank r simulates its own replica of the workload

@@ -22,6 +22,8 @@
 // results at 1.1 to 3.7 times the time over the measured sweeps -- 52.6 ms
 // against 19.2 ms for 10,000 x 1,000 requests under 7 runs, 273 ms against
 // 108 ms for 1,024 x 100,000 under 3 -- and nowhere less.)
+// While a queue head waits, FCFS and ISJL without a binding budget serve up to 32
+// completions in a pass (a batch).
 // Arrivals that cannot start anything before the next completion are released
 // at that completion, and an admission that starts several requests does so
 // up to 32 (ISJL plan entries: all) at a time, with the same outcome as one
@@ -29,11 +31,12 @@
 //
 // Layout.  Worker (batch slot) w lives in lane w % 32, register row w / 32,
 // so a warp holds B <= 32 * SPL workers.  Values that change only at events
-// (next arrival, start range, KV reservation) are kept as warp-uniform scalars.  The pending queue is a bitset over the instance's
-// request positions sorted by (o desc, index asc) -- the longest pending
-// request is the lowest set bit -- with a summary word per 32 words, in shared
-// memory.  ISJL plans are per-worker FIFO lists linked through a global
-// scratch array.
+// (next arrival, start range, KV reservation) are kept as warp-uniform scalars.
+// The pending queue is a bitset over the instance's request positions sorted by
+// (o desc, index asc) -- the longest pending request is the lowest set bit --
+// with a summary word per 32 words, in shared memory.  ISJL plans are per-worker
+// FIFO lists linked through a global scratch array.  Many instances of at most 32
+// requests go to tiny_kernel.cu instead (the rule is in launch_sim).
 #include <algorithm>
 #include <climits>
 #include <cstdint>

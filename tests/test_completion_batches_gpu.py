@@ -41,3 +41,19 @@ def test_batches_of_completions(S, O, policy, kind, B):  # noqa: F811
         if slack is not None:
             o = np.minimum(o, 65_535 - 40)
         run_both(S, O, a, p, o, B, [policy] * 2, [50, INF], kv, False, slack=slack, max_steps=ms)
+
+
+def test_budgets_around_the_longest_length(S, O):  # noqa: F811
+    """A budget of 65,535 or more never plans and never shuts the gate and has
+    a body of its own; 65,534 still can, with a request of 65,535 tokens."""
+    rng = np.random.default_rng(9)
+    o = lengths(rng, "long", (4, 60))
+    o[:, :3] = 65_535
+    o[1, 3:6] = 65_534
+    p = np.zeros_like(o)
+    a = np.zeros_like(o)
+    a[2:] = np.sort(rng.integers(0, 90_000, (2, 60)), axis=1)
+    for B in (2, 5, 40):
+        for pol in ("isjl", "isjl_beta"):
+            run_both(S, O, a, p, o, B, [pol] * 4, [65_533, 65_534, 65_535, INF], INF, False)
+            run_both(S, O, a, p, o, B, [pol] * 4, [65_533, 65_534, 65_535, INF], 150_000, False)
