@@ -57,3 +57,22 @@ def test_budgets_around_the_longest_length(S, O):  # noqa: F811
         for pol in ("isjl", "isjl_beta"):
             run_both(S, O, a, p, o, B, [pol] * 4, [65_533, 65_534, 65_535, INF], INF, False)
             run_both(S, O, a, p, o, B, [pol] * 4, [65_533, 65_534, 65_535, INF], 150_000, False)
+
+
+@pytest.mark.parametrize("kv", [INF, 30_000])
+@pytest.mark.parametrize("B", [3, 32, 100])
+def test_sjf_on_both_sides_of_its_queue_rule(S, O, kv, B):  # noqa: F811
+    """SJF has batches where the requests' tokens exceed 1.5 times what the slots
+    or the KV serve until the last arrival: last arrivals around that line, few
+    and many lengths, and more than 32 requests of the shortest one."""
+    rng = np.random.default_rng(17 + B)
+    n = 260
+    o = np.stack([rng.integers(1, 900, n), rng.integers(1, 900, n), rng.choice([90, 91, 92], n),
+                  np.full(n, 250), rng.integers(1, 5, n) * 100, rng.integers(1, 40, n)]).astype(np.int32)
+    served = np.minimum(B, kv * n // o.sum(axis=1, dtype=np.int64))
+    line = (2 * o.sum(axis=1, dtype=np.int64)) // (3 * served)
+    p = np.zeros_like(o)
+    for last in (line - 1, line, line + 1, line // 3):
+        a = np.sort(rng.random((6, n)) * last[:, None], axis=1).astype(np.int32)
+        a[:, -1] = last
+        run_both(S, O, a, p, o, B, ["sjf"], [0], kv, False)
