@@ -1292,9 +1292,11 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
                 near_end = INT_MIN;
             }
         };
+        // a pass costs two or three completions one at a time: none where the next
+        // arrival, which ends it, is nearer (a quarter or half of the span: the same times)
         auto waits = [&]() -> bool {
             if (P == ISJL_POLICY_FCFS) return fcfs < rel;
-            return pend > 0 && next_arr - k >= span >> 3;   // two or three completions before it
+            return pend > 0 && next_arr - k >= span >> 3;
         };
         auto batch = [&]() -> bool {
             if (skip > 0) { skip--; return false; }
@@ -1645,10 +1647,9 @@ constexpr int sim_min_blocks() {
 }
 
 // Whether SJF's body with batches of completions serves an instance.  It needs a
-// queue that lasts over several arrivals, while its loop is 13% longer (516
-// instructions a request against 454).  The line: the requests' tokens are more
-// than 1.5 times what the slots, or the requests of mean length that the KV holds,
-// serve until the last arrival.  1,500 x 701 requests of 1 to 1,999 tokens, without
+// queue that lasts over several arrivals; elsewhere its longer loop costs 6 to 12%.
+// The line: the requests' tokens are more than 1.5 times what the slots, or the
+// requests of mean length that the KV holds, serve until the last arrival.  1,500 x 701 requests of 1 to 1,999 tokens, without
 // -> with batches: B 200, at 0.67, 1 and 2 times 1.02 -> 1.14, 0.97 -> 1.07, 0.78 ->
 // 0.73 ms; B 16, 1.02 -> 1.12, 0.81 -> 0.86, 0.66 -> 0.60; at 3.3 (KV for 60) 0.83 ->
 // 0.66 and with all there at 0 0.77 -> 0.45 ms.
