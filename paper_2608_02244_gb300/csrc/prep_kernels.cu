@@ -376,6 +376,10 @@ summarize_kernel(const isjl_record *__restrict__ rec, int64_t n_inst, RunList ru
                  isjl_summary *out) {
     __shared__ FieldTotal part[kSumWarps][32];
     __shared__ FieldTotal blocks[kSumBlocks][32];           // the first block's is used
+    // a block's shared memory may be written by another only once it has started:
+    // every thread arrives here and waits before the stores; reading the records
+    // comes in between, so that the wait is over by then
+    asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");
     const int run = blockIdx.x / kSumBlocks, block = blockIdx.x % kSumBlocks;
     const int wid = threadIdx.x >> 5, f = threadIdx.x & 31;
     const int64_t *words = reinterpret_cast<const int64_t *>(rec + (int64_t)run * n_inst);
@@ -400,6 +404,7 @@ summarize_kernel(const isjl_record *__restrict__ rec, int64_t n_inst, RunList ru
     }
     part[wid][f] = t;
     __syncthreads();
+    asm volatile("barrier.cluster.wait;" ::: "memory");     // all blocks of the cluster run
     if (wid == 0) {
         for (int w = 1; w < kSumWarps; ++w) add_total(t, part[w][f], f);
         // the first block's shared memory, through the cluster
@@ -409,7 +414,8 @@ summarize_kernel(const isjl_record *__restrict__ rec, int64_t n_inst, RunList ru
         asm volatile("st.shared::cluster.b64 [%0], %1;" :: "r"(remote + 8), "l"(t.ok) : "memory");
         asm volatile("st.shared::cluster.b64 [%0], %1;" :: "r"(remote + 16), "l"(t.first_bad) : "memory");
     }
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    // (not .aligned: lanes of different fields have taken different branches)
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
     if (block != 0 || wid != 0) return;
     t = blocks[0][f];
     for (int b = 1; b < kSumBlocks; ++b) add_total(t, blocks[b][f], f);
