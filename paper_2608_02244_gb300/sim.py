@@ -25,8 +25,9 @@ KV_INF = 2**31 - 1
 MAX_B, MAX_LEN, MAX_RUNS = 512, 65535, 32
 FLAG_STEP_KERNEL, FLAG_EPOCH_KERNEL, FLAG_TIMING = 0, 1, 2
 
-# inputs of at most this many int32 in all go to the device in one copy: a copy
-# costs about 12 us of host time, packing them about 1 us per 10,000 values
+# inputs of at most this many int32 in all go to the device in one copy, and as many
+# results come back in one: a copy costs about 12 us of host time, packing the inputs
+# about 1 us per 10,000 values
 ONE_COPY_MAX = 1 << 17
 
 _I64 = ["T_make", "T_busy", "O", "Q", "W", "E", "token_adv", "sum_completion", "sum_latency",
@@ -265,7 +266,9 @@ class Simulator:
         self.n_inst, self.n, self.B = int(n_instances), int(n_per_instance), int(B)
         flags = (FLAG_EPOCH_KERNEL if epoch else FLAG_STEP_KERNEL) | (FLAG_TIMING if timing else 0)
         self.handle = isjl_sim_create(n_instances, n_per_instance, B, c, tau, p0, max_steps, flags)
-        self._block = None
+        self._records = None
+        self._per_req = None
+        self._block = None      # sweep()'s results on the device, never handed out
 
     def close(self):
         if self.handle:
@@ -279,18 +282,37 @@ class Simulator:
             pass
 
     def buffers(self, n_runs, per_request):
-        """Output tensors, views of one block kept between calls: records, then
-        start and completion steps."""
+        """Output tensors, kept between calls: a later call overwrites the records, a
+        later call with per-request outputs the start and completion steps too."""
+        torch = self.torch
+        need = n_runs * self.n_inst * RECORD_DTYPE.itemsize
+        if self._records is None or self._records.numel() < need:
+            self._records = torch.empty(need, dtype=torch.uint8, device="cuda")
+        rec = self._records[:need]
+        st = co = None
+        if per_request:
+            npr = n_runs * self.n_inst * self.n
+            if self._per_req is None or self._per_req[0].numel() < npr:
+                self._per_req = (torch.empty(npr, dtype=torch.int32, device="cuda"),
+                                 torch.empty(npr, dtype=torch.int32, device="cuda"))
+            st, co = self._per_req[0][:npr], self._per_req[1][:npr]
+        return rec, st, co
+
+    def _host_block(self, n_runs, per_request):
+        """Records, start and completion steps side by side in a block of sweep()'s
+        own, or None if they are more than one copy's worth."""
         torch = self.torch
         need = n_runs * self.n_inst * RECORD_DTYPE.itemsize
         per = 4 * n_runs * self.n_inst * self.n if per_request else 0
-        if self._block is None or self._block.numel() < need + 2 * per:
-            self._block = torch.empty(need + 2 * per, dtype=torch.uint8, device="cuda")
-        rec = self._block[:need]
+        total = need + 2 * per
+        if total > 4 * ONE_COPY_MAX:
+            return None
+        if self._block is None or self._block.numel() < total:
+            self._block = torch.empty(total, dtype=torch.uint8, device="cuda")
+        block = self._block[:total]
         if not per_request:
-            return rec, None, None
-        return (rec, self._block[need:need + per].view(torch.int32),
-                self._block[need + per:need + 2 * per].view(torch.int32))
+            return block, block, None, None
+        return block, block[:need], block[need:need + per].view(torch.int32), block[need + per:].view(torch.int32)
 
     def sweep_async(self, arrival, prompt, output, policies, deltas, kv_cap, per_request=False, stream=None,
                     counts=None, slack=None):
@@ -319,19 +341,27 @@ class Simulator:
         a, p, o = next(parts), next(parts), next(parts)
         cnt = next(parts) if counts is not None else None
         sl = next(parts) if slack is not None else None
-        rec, st, co = self.sweep_async(a, p, o, policies, deltas, kv_cap, per_request, stream, cnt, sl)
-        status, summ = isjl_sim_metrics(self.handle)
         R = len(policies)
+        block = self._host_block(R, per_request)
+        if block is None:
+            rec, st, co = self.sweep_async(a, p, o, policies, deltas, kv_cap, per_request, stream, cnt, sl)
+        else:
+            block, rec, st, co = block
+            _check(isjl_sim_run_sweep(self.handle, policies, deltas, kv_cap, a, p, o, rec, st, co, stream, cnt, sl),
+                   "isjl_sim_run_sweep")
+        status, summ = isjl_sim_metrics(self.handle)
+        if block is not None:                             # the outputs lie together: one copy
+            host = block.cpu()
+            rec = host[:rec.numel()]
+            if per_request:
+                st, co = host[rec.numel():].view(torch.int32).view(2, -1)
         out = {
-            "records": None,
+            "records": records_to_numpy(rec, R, self.n_inst),
             "summaries": [summary_to_dict(summ[i]) for i in range(R)],
             "status": status,
             "launches": isjl_sim_last_launches(self.handle),
         }
-        total = rec.numel() + (8 * st.numel() if per_request else 0)
-        host = self._block[:total].cpu().numpy()          # the outputs lie together: one copy
-        out["records"] = host[:rec.numel()].view(RECORD_DTYPE).reshape(R, self.n_inst)
         if per_request:
-            steps = host[rec.numel():].view(np.int32).reshape(2, R, self.n_inst, self.n)
-            out["start"], out["completion"] = steps[0], steps[1]
+            out["start"] = st.cpu().numpy().reshape(R, self.n_inst, self.n)
+            out["completion"] = co.cpu().numpy().reshape(R, self.n_inst, self.n)
         return out

@@ -1,0 +1,91 @@
+"""Which results of the device-resident call a later call on the same simulator
+may overwrite: records by records, start and completion steps by start and
+completion steps, and nothing by a call that returns host arrays of a few
+requests."""
+import types
+
+import numpy as np
+import pytest
+
+from conftest import cuda_available
+
+N, n = 5, 40
+TWO = (["fcfs", "isjl"], [0, 9])
+SEVEN = (["fcfs", "ljf", "isjl", "isjl", "isjl", "sjf", "isjl_beta"], [0, 0, 0, 9, 40, 0, 9])
+
+
+def span(t):
+    return t.data_ptr(), t.data_ptr() + t.numel() * t.element_size()
+
+
+def test_records_never_lie_over_steps():
+    """The output tensors alone, in host memory: no record of any call lies where
+    an earlier call's start or completion steps are."""
+    import torch
+    from paper_2608_02244_gb300 import sim
+    S = object.__new__(sim.Simulator)
+    S.n_inst, S.n, S.B, S.handle = N, n, 4, None
+    S._records = S._per_req = S._block = None
+    S.torch = types.SimpleNamespace(empty=lambda k, dtype, device: torch.empty(k, dtype=dtype),
+                                    uint8=torch.uint8, int32=torch.int32)
+    for runs in (1, 2, 7, 32):
+        _, st, co = S.buffers(runs, True)
+        assert span(st)[1] <= span(co)[0] or span(co)[1] <= span(st)[0]
+        assert st.numel() == co.numel() == runs * N * n and st.dtype == torch.int32
+        for later in (1, 2, 3, 7, 9, 32):
+            rec, none, _ = S.buffers(later, False)
+            assert none is None and rec.numel() == later * N * sim.RECORD_DTYPE.itemsize
+            for t in (st, co):
+                assert span(t)[1] <= span(rec)[0] or span(rec)[1] <= span(t)[0], (runs, later)
+
+
+@pytest.mark.gpu
+@pytest.mark.skipif(not cuda_available(), reason="needs a CUDA GPU")
+def test_steps_outlive_a_records_only_sweep():
+    import torch
+    from paper_2608_02244_gb300 import sim
+    rng = np.random.default_rng(4)
+    a = np.sort(rng.integers(0, 60, (N, n)), axis=1).astype(np.int32)
+    p = rng.integers(0, 9, (N, n)).astype(np.int32)
+    o = rng.integers(1, 70, (N, n)).astype(np.int32)
+    dev = [torch.from_numpy(x).cuda() for x in (a, p, o)]
+    S = sim.Simulator(N, n, 4)
+    try:
+        S.sweep_async(*dev, *SEVEN, 300, per_request=True)             # room for seven runs
+        rec, st, co = S.sweep_async(*dev, *TWO, 300, per_request=True)
+        start, completion = st.clone(), co.clone()
+        rec7, _, _ = S.sweep_async(*dev, *SEVEN, 300)
+        records = rec7.clone()
+        assert torch.equal(st, start) and torch.equal(co, completion)
+        assert torch.equal(rec7[:rec.numel()], rec)                    # records share a buffer
+        res = S.sweep(a, p, o, *TWO, 300, per_request=True)            # host arrays of a few requests
+        assert torch.equal(st, start) and torch.equal(co, completion) and torch.equal(rec7, records)
+        np.testing.assert_array_equal(res["start"].ravel(), start.cpu().numpy())
+        np.testing.assert_array_equal(res["completion"].ravel(), completion.cpu().numpy())
+    finally:
+        S.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.skipif(not cuda_available(), reason="needs a CUDA GPU")
+@pytest.mark.parametrize("shift", [-1, 0, 1])
+def test_host_arrays_on_both_sides_of_the_one_copy_line(shift):
+    """Outputs of up to ONE_COPY_MAX int32 come back in one copy, larger ones in
+    one per array: the same results."""
+    from paper_2608_02244_gb300 import sim
+    words = sim.RECORD_DTYPE.itemsize // 4
+    m = (sim.ONE_COPY_MAX // 2 - words) // 2 + shift      # 2 runs of words + 2 m int32
+    rng = np.random.default_rng(5)
+    o = rng.integers(1, 50, (1, m)).astype(np.int32)
+    z = np.zeros_like(o)
+    S = sim.Simulator(1, m, 64)
+    try:
+        both = S.sweep(z, z, o, *TWO, sim.KV_INF, per_request=True)
+        assert both["launches"] == 4 and both["status"] == 0
+        for i in range(2):
+            one = S.sweep(z, z, o, [TWO[0][i]], [TWO[1][i]], sim.KV_INF, per_request=True)
+            assert one["records"].tobytes() == both["records"][i].tobytes()
+            for f in ("start", "completion"):
+                assert one[f].shape == (1, 1, m) and (both[f][i] == one[f][0]).all() and (one[f] >= 0).all()
+    finally:
+        S.close()
