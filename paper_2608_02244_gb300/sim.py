@@ -328,16 +328,13 @@ class Simulator:
         completion (n_runs, n_inst, n) or None, per-run summaries, device status."""
         torch = self.torch
 
-        def dev(x):
-            t = torch.as_tensor(np.ascontiguousarray(x, dtype=np.int32)) if not torch.is_tensor(x) else x
-            return t.to(device="cuda", dtype=torch.int32).contiguous()
-
-        given = [x for x in (arrival, prompt, output, counts, slack) if x is not None]
+        given = [arrival, prompt, output] + [x for x in (counts, slack) if x is not None]
+        given = [x if torch.is_tensor(x) else np.ascontiguousarray(x, dtype=np.int32) for x in given]
         if all(isinstance(x, np.ndarray) for x in given) and sum(x.size for x in given) <= ONE_COPY_MAX:
-            flat = np.concatenate([np.asarray(x, dtype=np.int32).ravel() for x in given])
-            parts = iter(torch.from_numpy(flat).to("cuda").split([x.size for x in given]))
+            flat = torch.from_numpy(np.concatenate([x.ravel() for x in given]))
+            parts = iter(flat.to("cuda").split([x.size for x in given]))
         else:
-            parts = iter([dev(x) for x in given])
+            parts = iter([torch.as_tensor(x).to(device="cuda", dtype=torch.int32).contiguous() for x in given])
         a, p, o = next(parts), next(parts), next(parts)
         cnt = next(parts) if counts is not None else None
         sl = next(parts) if slack is not None else None

@@ -89,3 +89,18 @@ def test_host_arrays_on_both_sides_of_the_one_copy_line(shift):
                 assert one[f].shape == (1, 1, m) and (both[f][i] == one[f][0]).all() and (one[f] >= 0).all()
     finally:
         S.close()
+
+
+@pytest.mark.parametrize("missing", [0, 1, 2])
+def test_a_missing_input_is_refused(missing):
+    """The optional counts and slack must not take the place of an input that is
+    None: it is refused before anything reaches the device."""
+    from paper_2608_02244_gb300 import sim
+    import torch
+    S = object.__new__(sim.Simulator)
+    S.n_inst, S.n, S.B, S.handle, S.torch = N, n, 4, None, torch
+    S._records = S._per_req = S._block = None
+    x = np.ones((N, n), np.int32)
+    args = [None if i == missing else x for i in range(3)]
+    with pytest.raises(TypeError):
+        S.sweep(*args, *TWO, 300, counts=np.full(N, n, np.int32), slack=x)
