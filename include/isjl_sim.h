@@ -124,7 +124,8 @@ typedef struct {
     int64_t sum_extent;      /* sum over nonempty steps of max r - min r */
     int64_t max_extent;      /* max over steps of max r - min r */
     int64_t violations;      /* steps whose extent exceeds delta (0 for LJF and ISJL) */
-    int64_t kv_violations;   /* steps whose reserved KV exceeds kv_cap (always 0) */
+    int64_t kv_violations;   /* 0: every start is checked against kv_cap; 1 if the reserved KV exceeded it
+                                in some step all the same, which also makes status INTERNAL */
     int64_t peak_kv;         /* max reserved KV (sum of o over the running set) */
     int64_t peak_batch;      /* max |S| */
     int64_t status;          /* isjl_status of this run on this instance */

@@ -116,6 +116,12 @@ __device__ __forceinline__ int64_t task_status(const InstStats &is, int32_t kv_l
     return is.O + (int64_t)is.maxA + 1 >= (int64_t)(1 << 30) ? ISJL_ERR_INVALID_ARG : ISJL_OK;
 }
 
+// a run's status given its largest reservation so far: every start is checked
+// against the cap, so a reservation beyond it is a library bug
+__host__ __device__ __forceinline__ int64_t checked_status(int64_t status, int32_t peak_kv, int64_t kv_cap) {
+    return peak_kv > kv_cap ? ISJL_ERR_INTERNAL : status;
+}
+
 // what a simulation kernel counted for one task
 struct RecordTotals {
     int64_t W, E, sum_completion, sum_extent;
@@ -140,7 +146,7 @@ __device__ __forceinline__ void store_record(const SimArgs &A, const InstStats &
     R.sum_extent = t.sum_extent;
     R.max_extent = t.max_extent;
     R.violations = t.violations;
-    R.kv_violations = 0;   // every start keeps the reservation within the cap
+    R.kv_violations = t.peak_kv > A.kv_cap;   // (and then status is INTERNAL, see checked_status)
     R.peak_kv = t.peak_kv;
     R.peak_batch = t.peak_batch;
     R.status = t.status;

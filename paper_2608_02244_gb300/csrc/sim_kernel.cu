@@ -1590,7 +1590,7 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
             peakkv = __reduce_max_sync(kFull, peakkv);
             peakb = __reduce_max_sync(kFull, peakb);
         }
-        if (peakkv > kv_lim) status = ISJL_ERR_INTERNAL;   // every start checks its reservation
+        status = checked_status(status, peakkv, kv_lim);
         if (status == ISJL_OK) {
             tok = (int32_t)is.O;
             E = W - is.Q;

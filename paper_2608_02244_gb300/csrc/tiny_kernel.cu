@@ -153,7 +153,10 @@ __device__ __forceinline__ void tiny_task(const SimArgs &A, int64_t inst, int ru
                 s_sum += s;
             }
             const int nxt = min(c_min, evt);
-            if (nxt <= k || nxt == INT_MAX) { t.status = ISJL_ERR_INTERNAL; break; }
+            t.peak_kv = max(t.peak_kv, kv);
+            if (nxt <= k || nxt == INT_MAX) t.status = ISJL_ERR_INTERNAL;
+            t.status = checked_status(t.status, kv, kv_lim);
+            if (t.status != ISJL_OK) break;
             if (run_cnt > 0) {                                       // steps k .. nxt - 1
                 const int64_t L = nxt - k;
                 const int ext = s_hi - s_lo;
@@ -164,7 +167,6 @@ __device__ __forceinline__ void tiny_task(const SimArgs &A, int64_t inst, int ru
                 if (ext > alpha) t.violations += (int32_t)L;
                 t.T_busy += (int32_t)L;
                 t.token_adv += (int32_t)(run_cnt * L);
-                t.peak_kv = max(t.peak_kv, kv);
                 t.peak_batch = max(t.peak_batch, run_cnt);
             }
             k = nxt;
