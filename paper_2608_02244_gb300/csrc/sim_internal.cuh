@@ -118,8 +118,8 @@ __device__ __forceinline__ int64_t task_status(const InstStats &is, int32_t kv_l
 
 // a run's status given its largest reservation so far: every start is checked
 // against the cap, so a reservation beyond it is a library bug
-__host__ __device__ __forceinline__ int64_t checked_status(int64_t status, int32_t peak_kv, int64_t kv_cap) {
-    return peak_kv > kv_cap ? ISJL_ERR_INTERNAL : status;
+__host__ __device__ __forceinline__ int64_t checked_status(int64_t status, int32_t peak_kv, int32_t kv_lim) {
+    return peak_kv > kv_lim ? ISJL_ERR_INTERNAL : status;
 }
 
 // what a simulation kernel counted for one task
