@@ -116,6 +116,12 @@ __device__ __forceinline__ int64_t task_status(const InstStats &is, int32_t kv_l
     return is.O + (int64_t)is.maxA + 1 >= (int64_t)(1 << 30) ? ISJL_ERR_INVALID_ARG : ISJL_OK;
 }
 
+// the first step that a run of max_steps >= 1 steps does not serve (k > max_steps);
+// INT32_MAX, which no run reaches, for every bound beyond the step numbers
+__host__ __device__ __forceinline__ int32_t step_guard(int64_t max_steps) {
+    return (int32_t)min((uint64_t)max_steps + 1u, (uint64_t)INT32_MAX);   // (unsigned: max_steps may be INT64_MAX)
+}
+
 // a run's status given its largest reservation so far: every start is checked
 // against the cap, so a reservation beyond it is a library bug
 __host__ __device__ __forceinline__ int64_t checked_status(int64_t status, int32_t peak_kv, int32_t kv_lim) {

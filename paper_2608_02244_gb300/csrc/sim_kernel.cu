@@ -424,10 +424,10 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
         bool L1_started = true;
         bool broken = false;   // an internal invariant failed: stop without touching memory
         const int64_t max_steps = A.max_steps > 0 ? A.max_steps : is.O + (int64_t)is.maxA + 1;
-        const int32_t step_guard = (int32_t)min(max_steps + 1, (int64_t)INT_MAX);
+        const int32_t guard = step_guard(max_steps);
         // the next step at which something other than a completion happens: the
         // guard, a new kbase, an arrival or o_1's delay expiry
-        int32_t evt_base = min(step_guard, kSpan), evt = 0;
+        int32_t evt_base = min(guard, kSpan), evt = 0;
 
         // plan links: request and planning length of the entry after a request,
         // in one word when request indices fit 16 bits, else the index plus one
@@ -1541,7 +1541,7 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
                 k = nxt;
             }
             if (k >= min(evt, next_arr)) {
-                if (k >= step_guard) { status = ISJL_ERR_STEP_LIMIT; break; }   // k > max_steps
+                if (k >= guard) { status = ISJL_ERR_STEP_LIMIT; break; }   // k > max_steps
                 if (k >= evt_base) {                 // keep the keys' relative steps within 32 - SH bits
                     const uint32_t d = (uint32_t)(k - kbase) << SH;
                     if (SPL > 1) {
@@ -1552,7 +1552,7 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
                     if (key0 != kEmpty) key0 -= d;
                     kbase = k;
                     nn = 0;
-                    evt_base = (int32_t)min((int64_t)step_guard, (int64_t)k + kSpan);
+                    evt_base = (int32_t)min((int64_t)guard, (int64_t)k + kSpan);
                 }
                 if (k >= next_arr) release();
             }

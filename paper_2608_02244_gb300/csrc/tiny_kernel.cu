@@ -79,7 +79,7 @@ __device__ __forceinline__ void tiny_task(const SimArgs &A, int64_t inst, int ru
         int t0 = 0, d1 = 0;
         bool L1_started = true;
         const int64_t max_steps = A.max_steps > 0 ? A.max_steps : is.O + (int64_t)is.maxA + 1;
-        const int guard = (int)min(max_steps + 1, (int64_t)INT_MAX);
+        const int guard = step_guard(max_steps);
 
         auto start = [&](int p, int w) {
             const int e = perm[p], u = U[p];
