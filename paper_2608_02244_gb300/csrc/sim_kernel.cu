@@ -1614,14 +1614,11 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
             E = W - warp_sum64((int64_t)R_l - rest);
             tok = (int32_t)__reduce_add_sync(kFull, (unsigned)(tok_l - tok_rest));
             sumc = sums + (int64_t)__reduce_add_sync(kFull, (unsigned)tok_l) - warp_sum64(run_c);
-            if (co_out) {
-                __syncwarp();
+            __syncwarp();                              // what was written ahead and did not happen
 #pragma unroll 1
-                for (int i = lane; i < n; i += 32)
-                    if (status != ISJL_ERR_STEP_LIMIT || co_out[i] >= k) co_out[i] = -1;
-                if (st_out && status != ISJL_ERR_STEP_LIMIT)
-#pragma unroll 1
-                    for (int i = lane; i < n; i += 32) st_out[i] = -1;
+            for (int i = lane; i < n; i += 32) {
+                if (co_out && (status != ISJL_ERR_STEP_LIMIT || co_out[i] >= k)) co_out[i] = -1;
+                if (st_out && status != ISJL_ERR_STEP_LIMIT) st_out[i] = -1;
             }
         }
     }

@@ -104,3 +104,41 @@ def test_a_missing_input_is_refused(missing):
     args = [None if i == missing else x for i in range(3)]
     with pytest.raises(TypeError):
         S.sweep(*args, *TWO, 300, counts=np.full(N, n, np.int32), slack=x)
+
+
+@pytest.mark.gpu
+@pytest.mark.skipif(not cuda_available(), reason="needs a CUDA GPU")
+@pytest.mark.parametrize("copies", [1, 4000])                 # a warp and a thread per task
+@pytest.mark.parametrize("max_steps", [0, 25])
+def test_start_or_completion_steps_alone(copies, max_steps):
+    """Either array may be asked for without the other: every entry is written,
+    -1 for what did not start or finish, and the same as with both."""
+    import torch
+    from paper_2608_02244_gb300 import sim
+    rng = np.random.default_rng(8)
+    m = 21
+    o = np.tile(rng.integers(1, 40, (1, m)), (copies, 1)).astype(np.int32)
+    a = np.tile(np.sort(rng.integers(0, 50, (1, m)), axis=1), (copies, 1)).astype(np.int32)
+    counts = np.where(np.arange(copies) % 2, m, m - 4).astype(np.int32)
+    slack = rng.integers(0, 9, (copies, m)).astype(np.int32)
+    a, p, o, counts, slack = (torch.from_numpy(x).cuda() for x in (a, np.zeros_like(o), o, counts, slack))
+    R = len(SEVEN[0])
+    S = sim.Simulator(copies, m, 3, max_steps=max_steps)
+    try:
+        for sl in (None, slack):
+            got = []
+            for want in ((True, True), (True, False), (False, True)):
+                rec = torch.empty(R * copies * sim.RECORD_DTYPE.itemsize, dtype=torch.uint8, device="cuda")
+                st, co = (torch.full((R, copies, m), -7, dtype=torch.int32, device="cuda") if w else None for w in want)
+                rc = sim.isjl_sim_run_sweep(S.handle, *SEVEN, 100, a, p, o, rec, st, co, count=counts, slack=sl)
+                assert rc == sim.ISJL_OK
+                torch.cuda.synchronize()
+                got.append((rec, st, co))
+            (rec, st, co), (rec_s, st_s, _), (rec_c, _, co_c) = got
+            assert torch.equal(rec, rec_s) and torch.equal(rec, rec_c)
+            assert torch.equal(st, st_s) and torch.equal(co, co_c)
+            assert int(st.min()) == int(co.min()) == -1                    # the unused slots at least
+            if max_steps:
+                assert bool(((st >= 0) & (co == -1)).any()) and int(co.max()) <= max_steps
+    finally:
+        S.close()
