@@ -1504,7 +1504,6 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
             bool served = false;
             if (run_cnt == 0) {                                  // nothing runs: the steps up to evt are idle
                 if (P == ISJL_POLICY_FCFS ? fcfs == n : rel == n && pend == 0 && plan_left == 0) break;
-                if (evt >= (1 << 30) - 1) { status = ISJL_ERR_INTERNAL; break; }   // cannot progress
                 smin = smax;
                 Tb -= evt - k;
             } else {
@@ -1514,7 +1513,7 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
             if (!served) {
                 // ---- steps k .. nxt - 1
                 const uint32_t m = __reduce_min_sync(kFull, key0);
-                int32_t nxt = min(kbase + (int32_t)(m >> SH), evt);   // the next completion (none: beyond evt) or event
+                int32_t nxt = (int32_t)min((uint32_t)kbase + (m >> SH), (uint32_t)evt);   // the next completion (none: beyond evt) or event
                 const int32_t ext = smax - smin;                     // max r - min r
                 const uint32_t m0 = (uint32_t)(k - smin + 1);        // max r at step k
                 peakkv = max(peakkv, kv_sum);

@@ -58,3 +58,33 @@ def test_bounds_that_no_run_reaches(S, O, max_steps, copies):  # noqa: F811
     assert (run_both(S, O, *args, slack=slack)["records"]["status"] == S.ISJL_ERR_STEP_LIMIT).any()
     res = run_both(S, O, *args, slack=slack, max_steps=max_steps)
     assert (res["records"]["status"] == 0).all() and (res["completion"] >= 0).all()
+
+
+@pytest.mark.gpu
+@pytest.mark.skipif(not cuda_available(), reason="needs a CUDA GPU")
+@pytest.mark.parametrize("copies", [1, 4000])                 # a warp and a thread per task
+@pytest.mark.parametrize("max_steps", [0, 2**31 - 1])
+def test_idling_at_the_end_of_the_step_range(S, max_steps, copies):  # noqa: F811
+    """Predictions leave o_1's delay idle: packs planned with 2,000 tokens are done
+    after two, and o_1 waits 1,000 steps.  The same requests at step 0 and at the
+    last arrival that is accepted (sum o + max arrival = 2^30 - 2): every step is
+    the same number of steps later, under the default bound (which ends the run in
+    that idle time) and under one that no run reaches."""
+    o = np.ones((copies, 4), np.int32)
+    slack = np.tile(np.array([[4999, 3999, 999, 999]], np.int32), (copies, 1))
+    z = np.zeros_like(o)
+    late = 2**30 - 2 - int(o[0].sum())
+    pols, ds = ["isjl", "isjl_beta", "isjl", "sjf"], [1000, 1000, INF, 0]
+    sm = S.Simulator(copies, o.shape[1], 2, max_steps=max_steps)
+    try:
+        early = sm.sweep(z, z, o, pols, ds, INF, per_request=True, slack=slack)
+        res = sm.sweep(z + late, z, o, pols, ds, INF, per_request=True, slack=slack)
+    finally:
+        sm.close()
+    assert (early["records"]["status"][0] == (0 if max_steps else S.ISJL_ERR_STEP_LIMIT)).all()
+    assert max_steps == 0 or (early["records"]["T_make"][0] > 1000).all()
+    for f in ("status", "T_busy", "O", "Q", "W", "E", "token_adv", "sum_extent", "max_extent", "violations",
+              "peak_kv", "peak_batch"):
+        np.testing.assert_array_equal(res["records"][f], early["records"][f], err_msg=f)
+    for f in ("start", "completion"):
+        np.testing.assert_array_equal(res[f], np.where(early[f] < 0, -1, early[f] + late), err_msg=f)
