@@ -50,7 +50,9 @@ constexpr int32_t kNone = -1;
 // ISJL whose budget no request's length exceeds: it never plans (o_2 <= alpha) and
 // its gate never shuts, so it starts the longest pending request that fits
 constexpr int kPolicyLpt = ISJL_POLICY_ISJL_BETA + 1;
-constexpr int kPolicySjfQueue = ISJL_POLICY_ISJL_BETA + 2;   // SJF where a queue builds up: batches of completions
+// SJF and FCFS where a queue builds up (queue_builds_up): with batches of completions
+constexpr int kPolicySjfQueue = ISJL_POLICY_ISJL_BETA + 2;
+constexpr int kPolicyFcfsQueue = ISJL_POLICY_ISJL_BETA + 3;
 constexpr uint32_t kEmpty = 0xFFFFFFFFu;   // key of a slot that holds no running request
 
 // bits of a running request's key that hold its register row
@@ -280,7 +282,8 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
     constexpr bool kLpt = P == kPolicyLpt;
     constexpr bool kFar = SPL >= 16 && !kIsjl;
     constexpr bool kSjf = P == ISJL_POLICY_SJF || P == kPolicySjfQueue;
-    constexpr bool kBatch = P == ISJL_POLICY_FCFS || kLpt || P == kPolicySjfQueue;
+    constexpr bool kFcfs = P == ISJL_POLICY_FCFS || P == kPolicyFcfsQueue;
+    constexpr bool kBatch = P == kPolicyFcfsQueue || kLpt || P == kPolicySjfQueue;
     const int n_slots = A.n, B = A.B;
     const int64_t base = inst * (int64_t)n_slots;
     const InstStats is = A.inst[inst];
@@ -324,7 +327,7 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
     int32_t Tb = 0, tok = 0, maxext = 0, viol = 0, peakb = 0, Tmake = 0;
 
     if (status == ISJL_OK && n > 0) {
-        if (P != ISJL_POLICY_FCFS) {
+        if (!kFcfs) {
 #pragma unroll 1
             for (int w = lane; w < words0; w += 32) S.pend0[w] = 0u;
 #pragma unroll 1
@@ -379,7 +382,7 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
         auto load_window = [&]() {
             const int i = win_base + lane;
             win_a = i < n ? arr[i] : INT_MAX;
-            win_p = (i < n && P != ISJL_POLICY_FCFS) ? posof[i] : 0;
+            win_p = (i < n && !kFcfs) ? posof[i] : 0;
             if (kSjf) win_u = i < n ? oarr[i] : INT_MAX;
             // ask for the next 32 now, where instances are usually long enough to come
             // from memory (1,024 x 100,000 requests, B = 512: 39.5 -> 37.7 ms); with 8
@@ -401,7 +404,7 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
                 hw = (u << 16) | ((opaque(flags) & kSlack) ? (uint32_t)otru[i] : u);
             }
         };
-        if (P == ISJL_POLICY_FCFS) {
+        if (kFcfs) {
             load_heads();
             fh = __shfl_sync(kFull, hw, 0);
         }
@@ -584,7 +587,7 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
         };
         // requests with A_i <= k join the queue (a prefix: arrivals are non-decreasing)
         auto release = [&]() {
-            if (P != ISJL_POLICY_FCFS && rel == 0 && is.maxA <= k) {   // all of them at once
+            if (!kFcfs && rel == 0 && is.maxA <= k) {   // all of them at once
 #pragma unroll 1
                 for (int b = 0; b < words0; b += 32) {
                     const int i = b + lane;
@@ -603,7 +606,7 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
                 // released: window lanes at or after rel whose arrival is <= k (a prefix)
                 const bool ok = win_base + lane >= rel && win_a <= k;
                 const unsigned b = __ballot_sync(kFull, ok);
-                if (P != ISJL_POLICY_FCFS) {
+                if (!kFcfs) {
                     if (ok) {
                         atomicOr(&S.pend0[win_p >> 5], 1u << (win_p & 31));
                         atomicOr(&S.pend1[win_p >> 10], 1u << ((win_p >> 5) & 31));
@@ -1028,7 +1031,7 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
         auto admit = [&]() {
             bool blocked;
             int32_t next_fit = INT_MAX;
-            if (P == ISJL_POLICY_FCFS) {
+            if (kFcfs) {
                 // arrival order; the first request that does not fit ends the step;
                 // one at a time for the first two starts (usually all there are),
                 // then 32 at a time
@@ -1182,8 +1185,8 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
             nn = 0;
         };
 
-        // ---- Batches of completions (FCFS, SJF, and ISJL without a binding
-        // budget).  While the queue head waits for KV or a slot, nothing but completions
+        // ---- Batches of completions (ISJL without a binding budget, and FCFS and SJF
+        // where a queue builds up).  While the queue head waits for KV or a slot, nothing but completions
         // lets a request start (longest or shortest first: until the next arrival, which
         // may come before the head).  The next up to 32
         // completions (i, ascending) and the next up to 31 queued requests (j, in
@@ -1295,11 +1298,16 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
                 near_end = INT_MIN;
             }
         };
-        // a pass costs two or three completions one at a time: none where the next
-        // arrival, which ends it, is nearer (a quarter or half of the span: the same times)
+        // A pass costs two or three completions one at a time.  With few running each
+        // start completes before the others and a short queue is used up, so that a
+        // pass serves one or two: none with fewer than 5 running (longest first, 300 x
+        // 1,000 requests against one at a time: B = 3 0.8, B = 5 1.07, B = 6 1.14 times
+        // as fast) or 4 queued, and none where the next arrival, which ends it, is near
+        // (an eighth, a quarter or half of the span: the same times)
         auto waits = [&]() -> bool {
-            if (P == ISJL_POLICY_FCFS) return fcfs < rel;
-            return pend > 0 && next_arr - k >= span >> 3;
+            if (run_cnt < 5) return false;
+            if (kFcfs) return rel - fcfs >= 4;
+            return pend >= 4 && next_arr - k >= span >> 3;
         };
         auto batch = [&]() -> bool {
             if (skip > 0) { skip--; return false; }
@@ -1506,7 +1514,7 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
         for (;;) {
             bool served = false;
             if (run_cnt == 0) {                                  // nothing runs: the steps up to evt are idle
-                if (P == ISJL_POLICY_FCFS ? fcfs == n : rel == n && pend == 0 && plan_left == 0) break;
+                if (kFcfs ? fcfs == n : rel == n && pend == 0 && plan_left == 0) break;
                 smin = smax;
                 Tb -= evt - k;
             } else {
@@ -1647,18 +1655,28 @@ constexpr int sim_min_blocks() {
     return SPL >= 16 ? ISJL_SIM_BLOCKS16 : ISJL_SIM_MIN_BLOCKS;
 }
 
-// Whether SJF's body with batches of completions serves an instance.  It needs a
-// queue that lasts over several arrivals; elsewhere its longer loop costs 6 to 12%.
-// The line: the requests' tokens are more than 1.5 times what the slots, or the
-// requests of mean length that the KV holds, serve until the last arrival.  1,500 x 701 requests of 1 to 1,999 tokens, without
-// -> with batches: B 200, at 0.67, 1 and 2 times 1.02 -> 1.14, 0.97 -> 1.07, 0.78 ->
-// 0.73 ms; B 16, 1.02 -> 1.12, 0.81 -> 0.86, 0.66 -> 0.60; at 3.3 (KV for 60) 0.83 ->
-// 0.66 and with all there at 0 0.77 -> 0.45 ms.
-__device__ __forceinline__ bool sjf_queues(const SimArgs &A, int64_t inst) {
+// Whether FCFS's or SJF's body with batches of completions serves an instance.  It
+// pays where a queue lasts over many completions; elsewhere its size costs the single
+// events 8 to 20%.  `fit` requests of mean length fit the KV, `served` run at once, and
+// O / room is the load.  Simulation times of 300 x 1,000 requests, one at a time
+// divided by with batches:
+//   FCFS  slots bind: B = 256, load 0.9 0.9, 1.1 1.0 (n = 3,000 1.7), 1.5 1.2, 4 1.6;
+//         B = 16, load 0.9 0.8, 1.1 1.0, 1.5 1.2; B = 10 1.0, B = 6 0.9 at any load
+//         KV binds, so that the head waits earlier: B = 256, load 0.67 0.95 (n = 3,000
+//         1.6), 0.83 1.2 (2.6), 1 1.7; B = 32 0.96, 1.1, 1.2; n = 50, B = 32 1.0
+//   SJF   n = 400, load 1.5 0.87, 2 1.0, 4 1.1, all there at 0 1.8; n = 100 0.84, 0.95,
+//         1.1, 1.2; n = 50 0.80, 0.83, 0.98, 1.1
+// (Near a line the instances of one run take both bodies, which crowd each other out
+// of the instruction cache, the more the smaller n is: hence n >= 100, and the lines
+// lie above the point where both are the same.)
+__device__ __forceinline__ bool queue_builds_up(const SimArgs &A, int64_t inst, bool sjf) {
     const InstStats is = A.inst[inst];
     const int64_t kv = min(A.kv_cap, (int64_t)INT_MAX);
-    const int64_t served = min((int64_t)A.B, kv * is.n / max(is.O, (int64_t)1));
-    return 2 * is.O > 3 * served * max(is.maxA, 0);
+    const int64_t fit = kv * is.n / max(is.O, (int64_t)1), served = min((int64_t)A.B, fit);
+    const int64_t room = served * max(is.maxA, 0);         // tokens served until the last arrival
+    if (is.n < 100) return false;
+    if (sjf) return A.B >= 8 && is.O > 3 * room;
+    return served >= 16 && (fit < A.B ? 3 * is.O > 2 * room : is.O > room);
 }
 
 template <int SPL>
@@ -1690,10 +1708,13 @@ sim_kernel(SimArgs A, int64_t n_tasks) {
         const int64_t inst = t - (int64_t)turn * A.n_inst;
         const int run = A.runs.order[turn];
         switch (A.runs.policy[run]) {
-            case ISJL_POLICY_FCFS: run_task<SPL, ISJL_POLICY_FCFS>(A, S, lane, gwarp, inst, run); break;
+            case ISJL_POLICY_FCFS:
+                if (queue_builds_up(A, inst, false)) run_task<SPL, kPolicyFcfsQueue>(A, S, lane, gwarp, inst, run);
+                else run_task<SPL, ISJL_POLICY_FCFS>(A, S, lane, gwarp, inst, run);
+                break;
             case ISJL_POLICY_LJF:  run_task<SPL, ISJL_POLICY_LJF>(A, S, lane, gwarp, inst, run); break;
             case ISJL_POLICY_SJF:
-                if (sjf_queues(A, inst)) run_task<SPL, kPolicySjfQueue>(A, S, lane, gwarp, inst, run);
+                if (queue_builds_up(A, inst, true)) run_task<SPL, kPolicySjfQueue>(A, S, lane, gwarp, inst, run);
                 else run_task<SPL, ISJL_POLICY_SJF>(A, S, lane, gwarp, inst, run);
                 break;
             default:

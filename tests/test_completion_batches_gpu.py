@@ -59,20 +59,23 @@ def test_budgets_around_the_longest_length(S, O):  # noqa: F811
             run_both(S, O, a, p, o, B, [pol] * 4, [65_533, 65_534, 65_535, INF], 150_000, False)
 
 
-@pytest.mark.parametrize("kv", [INF, 30_000])
-@pytest.mark.parametrize("B", [3, 32, 100])
-def test_sjf_on_both_sides_of_its_queue_rule(S, O, kv, B):  # noqa: F811
-    """SJF has batches where the requests' tokens exceed 1.5 times what the slots
-    or the KV serve until the last arrival: last arrivals around that line, few
-    and many lengths, and more than 32 requests of the shortest one."""
+@pytest.mark.parametrize("policy, n", [("sjf", 260), ("sjf", 99), ("sjf", 100), ("fcfs", 260), ("fcfs", 99), ("fcfs", 100)])
+@pytest.mark.parametrize("kv", [INF, 30_000, 6_000])
+@pytest.mark.parametrize("B", [3, 7, 8, 15, 16, 32, 100])
+def test_both_sides_of_the_queue_rules(S, O, policy, n, kv, B):  # noqa: F811
+    """FCFS and SJF have batches from 100 requests on where their tokens are more
+    than some times what the slots or the KV serve until the last arrival: last
+    arrivals around each line, few and many lengths, and more than 32 requests of
+    the shortest one."""
     rng = np.random.default_rng(17 + B)
-    n = 260
     o = np.stack([rng.integers(1, 900, n), rng.integers(1, 900, n), rng.choice([90, 91, 92], n),
                   np.full(n, 250), rng.integers(1, 5, n) * 100, rng.integers(1, 40, n)]).astype(np.int32)
-    served = np.minimum(B, kv * n // o.sum(axis=1, dtype=np.int64))
-    line = (2 * o.sum(axis=1, dtype=np.int64)) // (3 * served)
+    O_ = o.sum(axis=1, dtype=np.int64)
+    fit = kv * n // O_
+    served = np.minimum(B, fit)
+    line = O_ // (3 * served) if policy == "sjf" else np.where(fit < B, 3 * O_ // (2 * served), O_ // served)
     p = np.zeros_like(o)
     for last in (line - 1, line, line + 1, line // 3):
         a = np.sort(rng.random((6, n)) * last[:, None], axis=1).astype(np.int32)
         a[:, -1] = last
-        run_both(S, O, a, p, o, B, ["sjf"], [0], kv, False)
+        run_both(S, O, a, p, o, B, [policy], [0], kv, False)
