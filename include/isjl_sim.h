@@ -49,7 +49,8 @@ typedef enum {
     ISJL_ERR_INFEASIBLE = 2,   /* some o_i < 1 or o_i > kv_cap: the request can never start */
     ISJL_ERR_OOM = 3,          /* device or pinned-host allocation failed in create / first host call */
     ISJL_ERR_CUDA = 4,         /* a CUDA runtime call failed (launch, copy, sync) */
-    ISJL_ERR_STEP_LIMIT = 5,   /* a simulation exceeded max_steps (defensive guard; never trapped) */
+    ISJL_ERR_STEP_LIMIT = 5,   /* a simulation reached max_steps or its default: partial counters, -1 for
+                                  requests that did not start or finish */
     ISJL_ERR_NOT_READY = 6,    /* metrics requested before any run */
     ISJL_ERR_INTERNAL = 7      /* an internal invariant of the simulation kernel failed (a library bug):
                                   the run stopped where it found it; its counters are partial and its
@@ -86,7 +87,9 @@ typedef struct {
     double c;                /* fixed cost of a nonempty step (paper: 0.0005) */
     double tau;              /* cost per unit of |S| * max r (paper: 1e-6) */
     double p0;               /* revenue per token (paper: 1/500) */
-    int64_t max_steps;       /* step guard per run; 0 = sum o + max arrival + 1 (a proven bound) */
+    int64_t max_steps;       /* step guard per run; 0 = sum o + max arrival + 1, which every run with exact
+                                lengths keeps; with slack ISJL may idle beyond it (o_1's delay is planned with
+                                upper bounds) and then ends with STEP_LIMIT: give a larger max_steps for those */
     uint32_t flags;          /* ISJL_FLAG_* */
 } isjl_config;
 
@@ -143,8 +146,8 @@ typedef struct {
  * run-major (record run * n_instances + inst).  start / completion: device
  * or NULL, n_runs * n_instances * n_per_instance int32 each, run-major; the
  * step a request started / completed, -1 for one that did not (an instance
- * with an error status, a run stopped by max_steps, the unused slots of a
- * ragged instance).  Output buffers are owned by the
+ * with an error status, a run that ends with STEP_LIMIT, by max_steps or with
+ * slack by its default, the unused slots of a ragged instance).  Output buffers are owned by the
  * caller and must stay valid until the run's work on the stream is done. */
 typedef struct {
     isjl_record *records;

@@ -47,12 +47,14 @@ inline int32_t run_beta(int32_t policy, int32_t delta) {
     return policy == ISJL_POLICY_ISJL_BETA ? isjl_beta(delta) : delta;
 }
 
-// the list of a sweep.  Runs with long tasks go first: SJF, then ISJL from the
-// largest budget down, FCFS, LJF (single runs of 10,000 x 1,000 requests: ISJL at
-// 1,024 / inf / 256 / 64 / 16 3.8 / 3.2 / 1.6 / 0.8 / 0.6 ms, FCFS 1.3, LJF 0.4).
-// All 7: 10.5 ms, in the caller's order 10.9; 1,500 x 701 under all policies
-// 1,180 us against 1,220, 3,000 x
-// 1,000 with predictions under 7 runs 3.3 ms against 3.8
+// the list of a sweep.  Runs with long tasks go first, so that short ones fill the
+// tail: SJF, then ISJL from the largest budget down, FCFS, LJF.  Single runs of
+// 10,000 x 1,000 requests: SJF 4.4 ms, ISJL at inf / 1,024 / 256 / 64 / 16 2.3 / 3.9 /
+// 1.8 / 1.0 / 0.8, FCFS 1.4, LJF 0.6.  All 7 but SJF take 9.40 ms, in the caller's
+// order 9.65; 3,000 x 1,000 with predictions under 7 runs 2.93 against 3.27, 1,500 x
+// 701 under all policies 0.95 against 0.96, 1,024 x 100,000 under 3 with B = 100 43
+// against 55.  By the single runs 1,024 would come before inf: measured too, that is
+// slower (9.71 and 3.17 ms)
 inline RunList run_list(int32_t n_runs, const int32_t *policies, const int32_t *deltas) {
     RunList r{};
     auto rank = [&](int32_t i) -> int64_t {
@@ -108,8 +110,8 @@ struct SimArgs {
 };
 
 // status of a task before it runs: the instance's, an infeasible length or an
-// instance beyond the step counter's range (every schedule ends by sum o + max
-// arrival; completion steps need < 2^30)
+// instance beyond the step counter's range (with exact lengths every schedule ends by
+// sum o + max arrival, with predictions the default step bound ends it there)
 __device__ __forceinline__ int64_t task_status(const InstStats &is, int32_t kv_lim) {
     if (is.status != ISJL_OK) return is.status;
     if (is.maxo > kv_lim) return ISJL_ERR_INFEASIBLE;

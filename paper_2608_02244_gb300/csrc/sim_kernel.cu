@@ -18,12 +18,10 @@
 // followed by steps that cannot either.  While LJF has a batch running or
 // ISJL's gate is shut, completions that do not change the running set's
 // earliest or latest start are served in the same pass (a completion window).
-// (A loop that advances every running request in every step gave the same
-// results at 1.1 to 3.7 times the time over the measured sweeps -- 52.6 ms
-// against 19.2 ms for 10,000 x 1,000 requests under 7 runs, 273 ms against
-// 108 ms for 1,024 x 100,000 under 3 -- and nowhere less.)
-// While a queue head waits, FCFS and ISJL without a binding budget serve up to 32
-// completions in a pass (a batch).
+// (Advancing every running request in every step takes 1.1 to 3.7 times as long
+// over the measured sweeps and nowhere less.)
+// While a queue head waits, ISJL without a binding budget, and FCFS and SJF where a
+// queue builds up, serve up to 32 completions in a pass (a batch).
 // Arrivals that cannot start anything before the next completion are released
 // at that completion, and an admission that starts several requests does so
 // up to 32 (ISJL plan entries: all) at a time, with the same outcome as one
@@ -232,9 +230,8 @@ __device__ __forceinline__ int first_pos_le(const int32_t *os, int n, int64_t x,
 // otherwise have the event loop compiled once for each of its outcomes, and the
 // copies crowd each other out of the instruction cache: a task runs most of its
 // code only a few times, so ISJL's runs are bound by instruction fetch.  (With
-// this, with short loops rolled and with one pass over the rows per completion
-// window, ISJL's body went from 104 to 76 KB; 100,000 x 500 requests under 5 runs
-// from 29.8 to 23.6 ms, the profit experiment from 3.56 to 2.57 ms.)
+// this and with short loops rolled: 100,000 x 500 requests under 5 runs 29.8 ->
+// 23.6 ms, the profit experiment 3.56 -> 2.57 ms.)
 __device__ __forceinline__ int opaque(int v) {
     asm volatile("" : "+r"(v));
     return v;
@@ -254,7 +251,6 @@ __device__ __forceinline__ int opaque(int v) {
 // the request leaves.
 // A started request runs uninterrupted, so its completion step is written out
 // when it starts.
-//
 //
 // What bounds it: issue of one dependent chain of warp-uniform instructions per
 // event (ncu: issue slots half busy, DRAM a few percent), so the column layout
@@ -280,7 +276,7 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
     constexpr int32_t kSpan = 1 << (30 - SH);       // kbase follows k when it is this far behind
     constexpr bool kIsjl = P == ISJL_POLICY_ISJL;
     constexpr bool kLpt = P == kPolicyLpt;
-    constexpr bool kFar = SPL >= 16 && !kIsjl;
+    constexpr bool kFar = SPL >= 16 && !kIsjl;      // prefetch (the reason is at load_window)
     constexpr bool kSjf = P == ISJL_POLICY_SJF || P == kPolicySjfQueue;
     constexpr bool kFcfs = P == ISJL_POLICY_FCFS || P == kPolicyFcfsQueue;
     constexpr bool kBatch = P == kPolicyFcfsQueue || kLpt || P == kPolicySjfQueue;
@@ -384,10 +380,11 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
             win_a = i < n ? arr[i] : INT_MAX;
             win_p = (i < n && !kFcfs) ? posof[i] : 0;
             if (kSjf) win_u = i < n ? oarr[i] : INT_MAX;
-            // ask for the next 32 now, where instances are usually long enough to come
-            // from memory (1,024 x 100,000 requests, B = 512: 39.5 -> 37.7 ms); with 8
-            // rows and less the two instructions and their registers cost the sweeps of
-            // 1,000 requests 2%
+            // ask for the next 32 now: with 16 rows few warps are resident, and long
+            // instances come from memory (whole sweep of 1,024 x 100,000 requests, B =
+            // 512: 44.4 -> 42.6 ms; short ones are in the cache anyway: 20,000 x 1,000
+            // 5.31 -> 5.27, x 200 4.15 -> 4.14).  With fewer rows other warps hide the
+            // wait and it only costs: B = 100, 1,024 x 100,000 43.3 -> 43.9
             if (kFar && lane < 2 && win_base + 32 < n) prefetch((lane ? posof : arr) + win_base + 32);
         };
         load_window();
@@ -1198,17 +1195,12 @@ __device__ __forceinline__ void run_task(const SimArgs &A, const WarpSmem &S, in
         // of these new requests would precede, where the known requests have all
         // started, and at evt.  The start range before each completion comes from
         // suffix minima and maxima over the batch and the range of all others.
-        // One event at a time, a completion with its start cost 0.42 us (FCFS over a
-        // 20,000-request trace); batched, 0.11 us.  FCFS alone, one at a time ->
-        // passes that end where the start range changes -> as here: 10,000 x 1,000
-        // requests 2.74 -> 1.33 -> 1.23 ms, 100,000 x 500 9.6 -> 5.1 -> 4.2 ms, the
-        // trace 8.35 -> 2.61 -> 2.16 ms.  Longest first, 10,000 x 1,000 requests: 4.6
-        // -> 3.25 -> 2.20 ms.  SJF, whose oldest request changes at nearly every
-        // completion, had none (0.90 -> 1.59 ms with passes that end there): 77 x 777
-        // requests 0.67 -> 0.38 ms.  ISJL with a binding
-        // budget has no such pass: its plan and gate leave few completions in a row
-        // (a pass for its plan entries, tried, made its body 15% larger and the sweeps
-        // 13 to 26% slower).
+        // One event at a time -> batched, simulation alone: FCFS over a 20,000-request
+        // trace 8.35 -> 2.16 ms (0.42 -> 0.11 us a request), 10,000 x 1,000 requests 2.74
+        // -> 1.23, 100,000 x 500 9.6 -> 4.2; longest first, 10,000 x 1,000 4.6 -> 2.2; SJF,
+        // 77 x 777 0.67 -> 0.38.  ISJL with a binding budget has no such pass: its plan
+        // and gate leave few completions in a row (a pass for its plan entries made its
+        // body 15% larger and the sweeps 13 to 26% slower).
 
         // collect the next completions: those within the next `span` steps, a number
         // of steps kept such that there are 16 to 32 where so many run
