@@ -40,7 +40,7 @@ def test_batches_of_completions(S, O, policy, kind, B):  # noqa: F811
                           (big + 40, rng.integers(0, 40, o.shape).astype(np.int32), 0), (big * 3, None, 997)]:
         if slack is not None:
             o = np.minimum(o, 65_535 - 40)
-        run_both(S, O, a, p, o, B, [policy] * 2, [50, INF], kv, False, slack=slack, max_steps=ms)
+        run_both(S, O, a, p, o, B, [policy] * 2, [50, INF], kv, slack=slack, max_steps=ms)
 
 
 def test_budgets_around_the_longest_length(S, O):  # noqa: F811
@@ -55,8 +55,8 @@ def test_budgets_around_the_longest_length(S, O):  # noqa: F811
     a[2:] = np.sort(rng.integers(0, 90_000, (2, 60)), axis=1)
     for B in (2, 5, 40):
         for pol in ("isjl", "isjl_beta"):
-            run_both(S, O, a, p, o, B, [pol] * 4, [65_533, 65_534, 65_535, INF], INF, False)
-            run_both(S, O, a, p, o, B, [pol] * 4, [65_533, 65_534, 65_535, INF], 150_000, False)
+            run_both(S, O, a, p, o, B, [pol] * 4, [65_533, 65_534, 65_535, INF], INF)
+            run_both(S, O, a, p, o, B, [pol] * 4, [65_533, 65_534, 65_535, INF], 150_000)
 
 
 @pytest.mark.parametrize("policy, n", [("sjf", 260), ("sjf", 99), ("sjf", 100), ("fcfs", 260), ("fcfs", 99), ("fcfs", 100)])
@@ -78,4 +78,4 @@ def test_both_sides_of_the_queue_rules(S, O, policy, n, kv, B):  # noqa: F811
     for last in (line - 1, line, line + 1, line // 3):
         a = np.sort(rng.random((6, n)) * last[:, None], axis=1).astype(np.int32)
         a[:, -1] = last
-        run_both(S, O, a, p, o, B, [policy], [0], kv, False)
+        run_both(S, O, a, p, o, B, [policy], [0], kv)

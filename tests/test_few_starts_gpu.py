@@ -24,9 +24,9 @@ def test_kv_around_a_few_of_the_longest(S, O, B):  # noqa: F811
     a = np.zeros_like(o)
     a[1] = np.sort(rng.integers(0, 100 * n // B, n))
     for kv in (100, 199, 200, 299, 300, 301, 400, INF):
-        run_both(S, O, a, p, o, B, *RUNS, kv, False)
+        run_both(S, O, a, p, o, B, *RUNS, kv)
     e = rng.integers(0, 40, o.shape).astype(np.int32)
-    run_both(S, O, a, p, o, B, *RUNS, 3 * 140 - 1, False, slack=e)
+    run_both(S, O, a, p, o, B, *RUNS, 3 * 140 - 1, slack=e)
 
 
 @pytest.mark.parametrize("burst", [1, 2, 3, 4])
@@ -40,4 +40,4 @@ def test_queues_of_a_few(S, O, burst, B):  # noqa: F811
     p = np.zeros_like(o)
     a = np.tile((np.arange(n) // burst * 50 * burst).astype(np.int32), (3, 1))
     for kv in (50, 120, INF):
-        run_both(S, O, a, p, o, B, *RUNS, kv, False)
+        run_both(S, O, a, p, o, B, *RUNS, kv)

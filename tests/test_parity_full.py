@@ -15,9 +15,8 @@ record.
       instance, so tests/golden/make_large_digest.py ran it once on all of them),
       and 8 spread-out instances against the oracle run here, field by field.
 
-Both kernel variants run; the oracle runs once, on every host core (a spawned
-process pool), and both are compared with it.  Integers bit-exact, fp64 within
-1e-12 relative; no record may carry the internal-error status.
+The oracle runs on every host core (a spawned process pool).  Integers bit-exact,
+fp64 within 1e-12 relative; no record may carry the internal-error status.
 """
 import time
 
@@ -50,8 +49,8 @@ def S():
     return sim
 
 
-def gpu_sweep(S, a, p, o, B, pols, ds, kv, epoch, per_request, counts=None, slack=None):
-    sm = S.Simulator(len(a), a.shape[1], B, epoch=epoch)
+def gpu_sweep(S, a, p, o, B, pols, ds, kv, per_request, counts=None, slack=None):
+    sm = S.Simulator(len(a), a.shape[1], B)
     try:
         res = sm.sweep(a, p, o, pols, ds, kv, per_request=per_request, counts=counts, slack=slack)
     finally:
@@ -68,17 +67,16 @@ def check_workload(S, pool, wid, pols, ds, per_request, sample=None):
     a, p, o, cnt, e = W.generate(wid, with_counts=True, with_slack=True)
     cnt = cnt if wl.ragged else None
     e = e if wl.robust else None
-    res = {ep: gpu_sweep(S, a, p, o, B, pols, ds, kv, ep, per_request, cnt, e) for ep in (False, True)}
+    r = gpu_sweep(S, a, p, o, B, pols, ds, kv, per_request, cnt, e)
     rows = np.arange(len(a)) if sample is None else np.asarray(sample)
     t = time.perf_counter()
     for i, (pol, d) in enumerate(zip(pols, ds)):
         rec, st, co = parallel.run(pool, pol, B, d, kv, a[rows], p[rows], o[rows], per_request=per_request,
                                    counts=None if cnt is None else cnt[rows], slack=None if e is None else e[rows])
-        for ep, r in res.items():
-            assert_records_equal(r["records"][i][rows], rec, f"w{wid} {pol} d={d} epoch={ep}")
-            if per_request:
-                np.testing.assert_array_equal(r["start"][i][rows], st, err_msg=f"w{wid} start {pol} {d} {ep}")
-                np.testing.assert_array_equal(r["completion"][i][rows], co, err_msg=f"w{wid} compl {pol} {d} {ep}")
+        assert_records_equal(r["records"][i][rows], rec, f"w{wid} {pol} d={d}")
+        if per_request:
+            np.testing.assert_array_equal(r["start"][i][rows], st, err_msg=f"w{wid} start {pol} {d}")
+            np.testing.assert_array_equal(r["completion"][i][rows], co, err_msg=f"w{wid} compl {pol} {d}")
     print(f"workload {wid}: {len(rows)} instances x {len(pols)} runs checked, oracle {time.perf_counter() - t:.0f} s")
 
 
@@ -116,7 +114,7 @@ def _golden_digest_module():
 
 
 def test_large_instance_every_instance_digest(S, pool):
-    """All 1,024 large instances, both kernels, against the oracle's digests.
+    """All 1,024 large instances against the oracle's digests.
     An instance whose generated inputs do not match the stored input digest
     (a platform whose floating-point draws differ) is checked against the
     oracle run here instead."""
@@ -139,19 +137,17 @@ def test_large_instance_every_instance_digest(S, pool):
     same = np.array([D.input_digest(a[i], p[i], o[i]) == stored[i][0] for i in range(wl.n_instances)])
     redo = np.flatnonzero(~same)
     t = time.perf_counter()
-    for ep in (False, True):
-        res = gpu_sweep(S, a, p, o, B, pols, ds, kv, ep, per_request=True)
-        rec, st, co = res["records"], res["start"], res["completion"]
-        bad = [i for i in np.flatnonzero(same)
-               if D.result_digest([rec[r][i] for r in range(len(pols))], [st[r][i] for r in range(len(pols))],
-                                  [co[r][i] for r in range(len(pols))]) != stored[i][1]]
-        assert not bad, f"epoch={ep}: {len(bad)} instances differ from the oracle, first {bad[:8]}"
-        for r, (pol, d) in enumerate(zip(pols, ds)):
-            if redo.size:
-                orec, ost, oco = parallel.run(pool, pol, B, d, kv, a[redo], p[redo], o[redo], per_request=True)
-                assert_records_equal(rec[r][redo], orec, f"w5 {pol} d={d} epoch={ep} (inputs drawn differently)")
-                np.testing.assert_array_equal(st[r][redo], ost)
-                np.testing.assert_array_equal(co[r][redo], oco)
-        del res, rec, st, co
+    res = gpu_sweep(S, a, p, o, B, pols, ds, kv, per_request=True)
+    rec, st, co = res["records"], res["start"], res["completion"]
+    bad = [i for i in np.flatnonzero(same)
+           if D.result_digest([rec[r][i] for r in range(len(pols))], [st[r][i] for r in range(len(pols))],
+                              [co[r][i] for r in range(len(pols))]) != stored[i][1]]
+    assert not bad, f"{len(bad)} instances differ from the oracle, first {bad[:8]}"
+    for r, (pol, d) in enumerate(zip(pols, ds)):
+        if redo.size:
+            orec, ost, oco = parallel.run(pool, pol, B, d, kv, a[redo], p[redo], o[redo], per_request=True)
+            assert_records_equal(rec[r][redo], orec, f"w5 {pol} d={d} (inputs drawn differently)")
+            np.testing.assert_array_equal(st[r][redo], ost)
+            np.testing.assert_array_equal(co[r][redo], oco)
     print(f"large instances: {int(same.sum())} by digest, {redo.size} by the oracle here, "
           f"{time.perf_counter() - t:.0f} s")

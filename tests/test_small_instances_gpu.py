@@ -23,9 +23,9 @@ def test_many_small_instances(S, O, n, B):  # noqa: F811
     counts = rng.integers(0, n + 1, N).astype(np.int32)
     slack = rng.integers(0, 6, (N, n)).astype(np.int32)
     big = 48
-    run_both(S, O, a, p, o, B, pols, ds, INF, False)
-    run_both(S, O, a, p, o, B, pols, ds, big, False, counts=counts, slack=slack)
-    run_both(S, O, a, p, o, B, pols, ds, 2 * big, False, max_steps=n + 9)
+    run_both(S, O, a, p, o, B, pols, ds, INF)
+    run_both(S, O, a, p, o, B, pols, ds, big, counts=counts, slack=slack)
+    run_both(S, O, a, p, o, B, pols, ds, 2 * big, max_steps=n + 9)
 
 
 @pytest.mark.parametrize("copies", [1, 4000])                 # a warp and a thread per task
@@ -36,7 +36,7 @@ def test_step_bound_with_predictions(S, O, copies):  # noqa: F811
     o = np.tile(np.array([[1, 8, 3, 2, 40, 41]], np.int32), (copies, 1))
     slack = np.tile(np.array([[5, 5, 3, 4, 3, 1]], np.int32), (copies, 1))
     z = np.zeros_like(o)
-    res = run_both(S, O, z, z, o, 3, ["isjl_beta"] * 2 + ["isjl"], [9, 9, 9], 48, False, slack=slack)
+    res = run_both(S, O, z, z, o, 3, ["isjl_beta"] * 2 + ["isjl"], [9, 9, 9], 48, slack=slack)
     assert (res["records"]["status"] == S.ISJL_ERR_STEP_LIMIT).any()
     assert (res["completion"] == -1).any()
 
@@ -49,4 +49,4 @@ def test_preparation_sizes(S, O, n):  # noqa: F811
     p = np.zeros_like(o)
     a = np.zeros_like(o)
     counts = np.array([n, max(1, n - 1), n // 2], np.int32)
-    run_both(S, O, a, p, o, 64, ["ljf", "sjf"], [0, 0], INF, False, counts=counts)
+    run_both(S, O, a, p, o, 64, ["ljf", "sjf"], [0, 0], INF, counts=counts)

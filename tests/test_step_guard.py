@@ -48,13 +48,13 @@ def test_bounds_that_no_run_reaches(S, O, max_steps, copies):  # noqa: F811
     a = np.tile(np.sort(rng.integers(0, 90, (1, 12)), axis=1), (copies, 1)).astype(np.int32)
     z = np.zeros_like(o)
     pols, ds = ["fcfs", "ljf", "sjf", "isjl", "isjl", "isjl_beta"], [0, 0, 0, 5, INF, 9]
-    res = run_both(S, O, a, z, o, 3, pols, ds, 100, False, max_steps=max_steps)
-    free = run_both(S, O, a, z, o, 3, pols, ds, 100, False, check=False)
+    res = run_both(S, O, a, z, o, 3, pols, ds, 100, max_steps=max_steps)
+    free = run_both(S, O, a, z, o, 3, pols, ds, 100, check=False)
     assert (res["records"]["status"] == 0).all() and res["records"].tobytes() == free["records"].tobytes()
     o = np.tile(np.array([[1, 8, 3, 2, 40, 41]], np.int32), (copies, 1))
     slack = np.tile(np.array([[5, 5, 3, 4, 3, 1]], np.int32), (copies, 1))
     z = np.zeros_like(o)
-    args = (z, z, o, 3, ["isjl_beta"] * 2 + ["isjl"], [9, 9, 9], 48, False)
+    args = (z, z, o, 3, ["isjl_beta"] * 2 + ["isjl"], [9, 9, 9], 48)
     assert (run_both(S, O, *args, slack=slack)["records"]["status"] == S.ISJL_ERR_STEP_LIMIT).any()
     res = run_both(S, O, *args, slack=slack, max_steps=max_steps)
     assert (res["records"]["status"] == 0).all() and (res["completion"] >= 0).all()

@@ -27,19 +27,17 @@ def _check_equal(g, r):
             np.testing.assert_array_equal(g[f], r[f], err_msg=f)
 
 
-@pytest.mark.parametrize("epoch", [False, True])
-def test_noalloc_matches_regular_sweep_twice(epoch):
+def test_noalloc_matches_regular_sweep_twice():
     import torch
     from paper_2608_02244_gb300 import sim, workloads as W
     cases = [
         (3, 24, 256, 200_000, ["fcfs", "ljf", "isjl", "isjl", "isjl"], [0, 0, 16, 256, INF]),
         (1, None, 32, 2048, ["fcfs", "ljf", "isjl"], [32, 32, 32]),
     ]
-    flags = sim.FLAG_EPOCH_KERNEL if epoch else sim.FLAG_STEP_KERNEL
     for wid, count, B, kv, pols, ds in cases:
         a_h, p_h, o_h = W.generate(wid, count)
         n_inst, n = a_h.shape
-        ref = sim.Simulator(n_inst, n, B, epoch=epoch)
+        ref = sim.Simulator(n_inst, n, B)
         try:
             want = ref.sweep(a_h, p_h, o_h, pols, ds, kv, per_request=True)
         finally:
@@ -49,7 +47,7 @@ def test_noalloc_matches_regular_sweep_twice(epoch):
             rec = torch.zeros(len(pols) * n_inst * sim.RECORD_DTYPE.itemsize, dtype=torch.uint8, device="cuda")
             st = torch.full((len(pols) * n_inst * n,), -7, dtype=torch.int32, device="cuda")
             co = torch.full_like(st, -7)
-            rc = sim.isjl_sim_run_sweep_noalloc(n_inst, n, B, pols, ds, kv, a, p, o, rec, st, co, flags=flags)
+            rc = sim.isjl_sim_run_sweep_noalloc(n_inst, n, B, pols, ds, kv, a, p, o, rec, st, co)
             assert rc == sim.ISJL_OK, sim.isjl_status_string(rc)
             torch.cuda.synchronize()
             got = sim.records_to_numpy(rec, len(pols), n_inst)
@@ -59,15 +57,13 @@ def test_noalloc_matches_regular_sweep_twice(epoch):
             np.testing.assert_array_equal(co.cpu().numpy().reshape(len(pols), n_inst, n), want["completion"])
 
 
-@pytest.mark.parametrize("epoch", [False, True])
-def test_noalloc_fewer_blocks_and_slack(epoch):
+def test_noalloc_fewer_blocks_and_slack():
     """Large instances (n = 100,000): the fixed array holds the plan scratch of
     fewer simulation blocks than are resident, so the call runs on fewer
     warps; and a robust workload, whose true lengths take 4 more bytes per
     request.  Both must match the regular sweep, records and per-request steps."""
     import torch
     from paper_2608_02244_gb300 import sim, workloads as W
-    flags = sim.FLAG_EPOCH_KERNEL if epoch else sim.FLAG_STEP_KERNEL
     cases = [(5, 3, 512, 1_000_000, ["fcfs", "isjl"], [0, 256], False),
              (8, 12, 256, 200_000, ["fcfs", "ljf", "isjl", "isjl"], [0, 0, 64, INF], True)]
     for wid, count, B, kv, pols, ds, robust in cases:
@@ -77,7 +73,7 @@ def test_noalloc_fewer_blocks_and_slack(epoch):
         if wid == 5:   # the plan scratch of the resident blocks does not fit: fewer blocks run
             free = (64 << 20) - n_inst * n * 20 - 4096
             assert free // (4 * n) < 4 * 152
-        ref = sim.Simulator(n_inst, n, B, epoch=epoch)
+        ref = sim.Simulator(n_inst, n, B)
         try:
             want = ref.sweep(a_h, p_h, o_h, pols, ds, kv, per_request=True, slack=e_h)
         finally:
@@ -87,7 +83,7 @@ def test_noalloc_fewer_blocks_and_slack(epoch):
         rec = torch.zeros(len(pols) * n_inst * sim.RECORD_DTYPE.itemsize, dtype=torch.uint8, device="cuda")
         st = torch.full((len(pols) * n_inst * n,), -7, dtype=torch.int32, device="cuda")
         co = torch.full_like(st, -7)
-        rc = sim.isjl_sim_run_sweep_noalloc(n_inst, n, B, pols, ds, kv, a, p, o, rec, st, co, flags=flags, slack=e)
+        rc = sim.isjl_sim_run_sweep_noalloc(n_inst, n, B, pols, ds, kv, a, p, o, rec, st, co, slack=e)
         assert rc == sim.ISJL_OK, sim.isjl_status_string(rc)
         torch.cuda.synchronize()
         got = sim.records_to_numpy(rec, len(pols), n_inst)
