@@ -347,18 +347,21 @@ class Simulator:
             _check(isjl_sim_run_sweep(self.handle, policies, deltas, kv_cap, a, p, o, rec, st, co, stream, cnt, sl),
                    "isjl_sim_run_sweep")
         status, summ = isjl_sim_metrics(self.handle)
-        if block is not None:                             # the outputs lie together: one copy
-            host = block.cpu()
-            rec = host[:rec.numel()]
+        if block is None:
+            records, steps = records_to_numpy(rec, R, self.n_inst), None
             if per_request:
-                st, co = host[rec.numel():].view(torch.int32).view(2, -1)
+                steps = [x.cpu().numpy().reshape(R, self.n_inst, self.n) for x in (st, co)]
+        else:                                             # the outputs lie together: one copy
+            host = block.cpu().numpy()
+            records = host[:rec.numel()].view(RECORD_DTYPE).reshape(R, self.n_inst)
+            if per_request:
+                steps = host[rec.numel():].view(np.int32).reshape(2, R, self.n_inst, self.n)
         out = {
-            "records": records_to_numpy(rec, R, self.n_inst),
+            "records": records,
             "summaries": [summary_to_dict(summ[i]) for i in range(R)],
             "status": status,
             "launches": isjl_sim_last_launches(self.handle),
         }
         if per_request:
-            out["start"] = st.cpu().numpy().reshape(R, self.n_inst, self.n)
-            out["completion"] = co.cpu().numpy().reshape(R, self.n_inst, self.n)
+            out["start"], out["completion"] = steps
         return out
